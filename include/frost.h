@@ -101,7 +101,13 @@ typedef struct {
                                the mixed mode, the time-step pass of a set of at least 8192
                                particles evaluates each pair once for both particles (the same
                                result bits: the pair criteria are symmetric and a minimum does
-                               not depend on the order).  1: all always; -1: never */
+                               not depend on the order).  1: all always; -1: never.  (Mixed mode,
+                               contexts of at least 16384 particles: frost_step orders the
+                               particles in space before every top-level step, and the time-step
+                               passes of large ordered lists, and of lists of at least 16384
+                               particles given to frost_timesteps, look at far groups of
+                               particles through bounds instead, again with the same bits; not
+                               with the exact fly-by derivative.) */
 } frost_opts;
 
 typedef enum {
@@ -121,7 +127,7 @@ void frost_default_opts(frost_opts *opt);
  * v[n][3] (host or device; copied), Newton's constant G and accuracy parameter eta
  * (eta = eta_ff = eta_fb, Sec. 4.3).  opt may be NULL for the defaults.  n >= 1 and
  * n < 2^31.  Non-finite inputs or non-positive masses give FROST_ENONFINITE / FROST_EINVAL.
- * The context allocates about (330 + 32 * levels_used) bytes per particle of device memory,
+ * The context allocates about (360 + 32 * levels_used) bytes per particle of device memory,
  * plus about 350 bytes per particle for each hierarchy level above the subtree threshold
  * whose FSI steps run on a stream of their own (frost_opts.branch_streams, allocated on
  * first use).

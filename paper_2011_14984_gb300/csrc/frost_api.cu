@@ -104,6 +104,13 @@ constexpr int64_t kSymCrossPrepassMinPairs = int64_t(1) << 26;
 // B-side reduction and dominant-term ballots cost what the saved pair bodies save)
 constexpr int64_t kSymGradMaxPairs = int64_t(1) << 23;
 
+// mixed mode: sets from this size on are put in spatial order (a frost_step call: all particles
+// at the top of every step, so that every list of the recursion inherits the order; the pass
+// entry points: the caller's list) and take the tile kernels of tile_kernels.cu; inside a step
+// the ordered lists of at least kTileMinN particles do
+constexpr int kOrderMinN = 16384;
+constexpr int kTileMinN = 8192;
+
 // autotuner rows: the pass kinds, and the Newtonian pass that feeds a gradient (mixed mode:
 // its wmax prepass and deferred double-float terms give it a cost profile of its own)
 constexpr int TUNE_ACC_ACCURATE = 3;
@@ -180,6 +187,11 @@ struct frost_ctx {
     std::vector<int32_t *> lvS, lvF;                 // per-level slow/fast lists
     unsigned *jbest = nullptr;                       // j-side minima of the symmetric time-step pass
     int *pblk = nullptr;                             // per-block slow counts of the partition
+    // spatial order (mixed mode, N >= kOrderMinN): workspace of the sort, the order of all
+    // particles of a step, and the positions and sorted list of a pass entry point's list
+    OrderWork ow;
+    int32_t *ord = nullptr, *opos = nullptr, *olist = nullptr;
+    bool ordered = false;                            // the lists of the running step are ordered
     double *pj = nullptr;                            // j-side partials of the symmetric pass
     size_t pj_elems = 0;
     double *part_hot2 = nullptr;                     // B-side hot-source partials of the
@@ -413,6 +425,20 @@ void pack_pos(frost_ctx *c, Lane &L, const int32_t *list, int n, void *rec)
 
 int badbit(const frost_ctx *c) { return c->eps2 == 0.0 ? ERR_COINCIDENT : ERR_NONFINITE; }
 
+// whether an entry point puts a list of n particles in spatial order
+bool use_order(const frost_ctx *c, int n) { return c->ord && n >= kOrderMinN; }
+
+void order_list(frost_ctx *c, const int32_t *list, int n, int32_t *pos, int32_t *sorted)
+{
+    launch_spatial_order(c->stream, list, n, c->x, c->N, c->ow, pos, sorted);
+    c->st.kernel_launches += 4;
+}
+
+// whether the time-step pass of a list of the running step takes the tile kernels.  The exact
+// fly-by derivative does not: its bound needs |v_ij| > 10 B eta |a_ij|, which with the largest
+// |a| of a tile fails for most of them (20 against 7 ms at 65536 particles)
+bool tile_tstep(const frost_ctx *c, int n) { return c->ordered && n >= kTileMinN && !(c->sym & FROST_FLYBY_EXACT); }
+
 // Newtonian accelerations of A from B (self: the same list); writes G * sum into out_soa
 // ([3][nA]) and, if given, out_aos ([nA][3]).  With wmax (mixed mode), also the weight
 // max_j m_j / r^3 of each particle's dominant term, which the following gradient pass uses.
@@ -564,14 +590,27 @@ void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA
     c->st.grad_pairs += pairs;
 }
 
-// symmetrised time-steps of the set P into tau[nP]
-void pass_tstep(frost_ctx *c, Lane &L, const int32_t *P, int nP, double *tau)
+// symmetrised time-steps of the set P into tau[nP].  tiled: P is in spatial order and takes the
+// tile kernels (mixed mode, main lane); pos (tiled only): tau[pos[k]] belongs to P[k].
+void pass_tstep(frost_ctx *c, Lane &L, const int32_t *P, int nP, double *tau, bool tiled = false,
+                const int32_t *pos = nullptr)
 {
     if (nP <= 0) return;
     if (nP == 1) {
         // no pair: with zero splits the finalisation writes eta * (+inf)
         launch_finalize_tau(L.s, L.part, 0, 1, c->eta, tau, &c->dmisc->err);
         c->st.kernel_launches += 1;
+        return;
+    }
+    const int64_t pairs = (int64_t)nP * (nP - 1);
+    if (tiled) {
+        {
+            TimedScope ts(c, L.s, PASS_TSTEP, pairs);
+            launch_tstep_tile(L.s, P, nP, c->x, c->v, c->m, c->N, c->G, c->eta, c->sym, c->n_sm, L.recA, c->jbest, pos,
+                              tau, &c->dmisc->err);
+        }
+        c->st.kernel_launches += 4;
+        c->st.tstep_pairs += pairs;
         return;
     }
     // exact fly-by derivative: the accelerations of the set due to itself, packed with the records
@@ -582,7 +621,6 @@ void pass_tstep(frost_ctx *c, Lane &L, const int32_t *P, int nP, double *tau)
     }
     if (c->mixed) launch_pack_tstep_mixed(L.s, P, nP, c->x, c->v, c->m, c->N, c->G, (float4 *)L.recA, acc);
     else launch_pack_tstep_fp64(L.s, P, nP, c->x, c->v, c->m, c->N, c->G, (double4_32a *)L.recA, acc);
-    const int64_t pairs = (int64_t)nP * (nP - 1);
     // mixed mode, large sets (or always with sym_cross = 1): every pair once for both particles
     if (c->mixed && &L == &c->main && (c->sym_cross > 0 || (c->sym_cross == 0 && nP >= kSymTstepMinN))) {
         const TstepSymShape sh = tstep_sym_shape(nP, c->n_sm, c->part_elems);
@@ -1020,7 +1058,7 @@ frost_status hhs_head(frost_ctx *c, const int32_t *P, int nP, double tau, int de
     }
     FROST_TRY(ensure_level(c, depth));
     Lane &M = c->main;
-    pass_tstep(c, M, P, nP, c->tau);
+    pass_tstep(c, M, P, nP, c->tau, tile_tstep(c, nP));
     launch_partition(M.s, P, nP, c->tau, tau, c->lvS[depth], c->lvF[depth], c->dmisc->counts, c->pblk);
     c->st.kernel_launches += nP >= PART_MULTI_MIN ? 2 : 1;
     h.done = false;
@@ -1156,7 +1194,8 @@ void destroy(frost_ctx *c)
     if (c->d_ecl) cudaFree(c->d_ecl);
     void *dev[] = {c->x, c->v, c->m, c->all, c->marks, c->recA, c->recB, c->part,
                    c->aA, c->aB, c->atA, c->atB, c->aC, c->tau, c->wA, c->wB, c->perm,
-                   c->ptmp, c->dmisc, c->hist, c->hA, c->hB, c->part_hot, c->part_hot2, c->pcnt, c->pj, c->jbest, c->pblk};
+                   c->ptmp, c->dmisc, c->hist, c->hA, c->hB, c->part_hot, c->part_hot2, c->pcnt, c->pj, c->jbest, c->pblk,
+                   c->ow.key, c->ow.key2, c->ow.pos2, c->ow.hist, c->opos, c->olist, c->ord};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (c->hmisc) cudaFreeHost(c->hmisc);
@@ -1305,6 +1344,15 @@ static frost_status init_impl(frost_ctx **out, int64_t n, const double *m, const
     if (c->mixed) INIT_CUDA(cudaMalloc(&c->pcnt, (c->pj_elems / 3) * SYM_PCNT_WARPS));
     INIT_CUDA(cudaMalloc(&c->jbest, sizeof(unsigned) * N));
     INIT_CUDA(cudaMalloc(&c->pblk, sizeof(int) * (size_t)partition_blocks((int)N)));
+    if (c->mixed && n >= kOrderMinN) {
+        INIT_CUDA(cudaMalloc(&c->ow.key, sizeof(unsigned) * N));
+        INIT_CUDA(cudaMalloc(&c->ow.key2, sizeof(unsigned) * N));
+        INIT_CUDA(cudaMalloc(&c->ow.pos2, sizeof(int32_t) * N));
+        INIT_CUDA(cudaMalloc(&c->ow.hist, sizeof(int) * (size_t)order_blocks((int)N) * ORDER_DIGITS));
+        INIT_CUDA(cudaMalloc(&c->opos, sizeof(int32_t) * N));
+        INIT_CUDA(cudaMalloc(&c->olist, sizeof(int32_t) * N));
+        INIT_CUDA(cudaMalloc(&c->ord, sizeof(int32_t) * N));
+    }
     INIT_CUDA(cudaMalloc(&c->perm, sizeof(int32_t) * N));
     INIT_CUDA(cudaMalloc(&c->ptmp, sizeof(int32_t) * N));
     if (n_clusters > 0) {
@@ -1553,7 +1601,12 @@ frost_status frost_timesteps(frost_ctx *c, const int32_t *set, int64_t n_set, do
     FROST_TRY(check_sizes(c, n_set, "n_set"));
     if (n_set > 0 && !tau) return fail(FROST_EINVAL, "tau is NULL");
     FROST_TRY(check_list(c, set, (int)n_set));
-    pass_tstep(c, c->main, set ? set : c->all, (int)n_set, tau);
+    if (use_order(c, (int)n_set) && !(c->sym & FROST_FLYBY_EXACT)) {
+        order_list(c, set, (int)n_set, c->opos, c->olist);
+        pass_tstep(c, c->main, c->olist, (int)n_set, tau, true, c->opos);
+    } else {
+        pass_tstep(c, c->main, set ? set : c->all, (int)n_set, tau);
+    }
     FROST_CUDA(cudaGetLastError());
     return sync_misc(c);
 }
@@ -1628,7 +1681,7 @@ frost_status hold2(frost_ctx *c, const int32_t *P, int nP, double tau, int depth
     }
     FROST_TRY(ensure_level(c, depth));
     int32_t *S = c->lvS[depth], *F = c->lvF[depth];
-    pass_tstep(c, c->main, P, nP, c->tau);
+    pass_tstep(c, c->main, P, nP, c->tau, tile_tstep(c, nP));
     launch_partition(c->stream, P, nP, c->tau, tau, S, F, c->dmisc->counts, c->pblk);
     c->st.kernel_launches += nP >= PART_MULTI_MIN ? 2 : 1;
     FROST_TRY(sync_misc(c));
@@ -1742,8 +1795,15 @@ frost_status frost_step(frost_ctx *c, double dt_pivot, int64_t n_steps)
     if (n_steps < 0) return fail(FROST_EINVAL, "n_steps < 0");
     if (c->n_clusters > 0) return batch_step(c, dt_pivot, n_steps);
     for (int64_t k = 0; k < n_steps; ++k) {
-        if (c->integrator == FROST_HOLD2) FROST_TRY(hold2(c, c->all, c->N, dt_pivot, 0));
-        else FROST_TRY(hhs_fsi(c, c->all, c->N, dt_pivot, 0));
+        // the order of this step's lists, from the present positions alone (a restarted run has
+        // the same order, and so the same bits, as an uninterrupted one)
+        c->ordered = use_order(c, c->N);
+        if (c->ordered) order_list(c, nullptr, c->N, c->opos, c->ord);
+        const int32_t *P = c->ordered ? c->ord : c->all;
+        const frost_status st =
+            c->integrator == FROST_HOLD2 ? hold2(c, P, c->N, dt_pivot, 0) : hhs_fsi(c, P, c->N, dt_pivot, 0);
+        c->ordered = false;
+        FROST_TRY(st);
         c->t += dt_pivot;
     }
     FROST_CUDA(cudaGetLastError());

@@ -255,6 +255,26 @@ void launch_wmax_sym_self(cudaStream_t s, const void *rec, int n, double eps2, i
 void launch_wmax_sym_cross(cudaStream_t s, const void *recA, int nA, const void *recB, int nB, double eps2, int n_sm,
                            float *wA, float *wB);
 
+// ---- spatially ordered lists (order_kernels.cu, tile_kernels.cu) -------------------------
+constexpr int ORDER_CHUNK = 2048;   // entries per block of the sort
+constexpr int ORDER_DIGITS = 2048;  // counts per block
+inline int order_blocks(int n) { return (n + ORDER_CHUNK - 1) / ORDER_CHUNK; }
+struct OrderWork {
+    unsigned *key = nullptr, *key2 = nullptr;  // [n] each
+    int32_t *pos2 = nullptr;                   // [n]
+    int *hist = nullptr;                       // [order_blocks(n) * ORDER_DIGITS]
+};
+// sorted[k] = list[pos[k]] (list NULL: the identity), neighbours in the list near in space;
+// a function of the members' positions and their order in the list alone
+void launch_spatial_order(cudaStream_t s, const int32_t *list, int n, const double *x, int N, const OrderWork &w,
+                          int32_t *pos, int32_t *sorted);
+// Mixed time-step pass of one spatially ordered set (any order gives the same result, the same
+// bits as launch_tstep): tau[pos[k]] (pos NULL: tau[k]) of list[k].  sym: 0..2 (not the exact
+// fly-by derivative); rec: 72 B per particle; best: [n] scratch
+void launch_tstep_tile(cudaStream_t s, const int32_t *list, int n, const double *x, const double *v, const double *m,
+                       int N, double G, double eta, int sym, int n_sm, void *rec, unsigned *best, const int32_t *pos,
+                       double *tau, int *err);
+
 // ---- single-CTA subtree solver (subtree.cu) ------------------------------------------
 constexpr int SUBTREE_MAX_FRAMES = 64;  // recursion frames per block (max_depth < 64)
 constexpr int SUBTREE_STAT_LEVELS = 48; // per-depth statistics (last entry: deeper levels)
