@@ -110,6 +110,10 @@ constexpr int64_t kSymGradMaxPairs = int64_t(1) << 23;
 // the ordered lists of at least kTileMinN particles do
 constexpr int kOrderMinN = 16384;
 constexpr int kTileMinN = 8192;
+// the same for the Newtonian and gradient passes: the lists of a pass entry point from
+// kOrderForceMinN particles on, and inside a step two lists of at least kTileForceMinN
+constexpr int kOrderForceMinN = 24576;
+constexpr int kTileForceMinN = 2048;
 
 // autotuner rows: the pass kinds, and the Newtonian pass that feeds a gradient (mixed mode:
 // its wmax prepass and deferred double-float terms give it a cost profile of its own)
@@ -439,19 +443,38 @@ void order_list(frost_ctx *c, const int32_t *list, int n, int32_t *pos, int32_t 
 // |a| of a tile fails for most of them (20 against 7 ms at 65536 particles)
 bool tile_tstep(const frost_ctx *c, int n) { return c->ordered && n >= kTileMinN && !(c->sym & FROST_FLYBY_EXACT); }
 
+// whether the Newtonian and gradient passes between two lists (or of one) of the running call take
+// the tile kernels
+bool tile_force(const frost_ctx *c, int nA, int nB) { return c->ordered && std::min(nA, nB) >= kTileForceMinN; }
+
+TileArgs tile_args(const frost_ctx *c, const Lane &L, const void *irec, int nA, const void *jrec, int nB, bool self)
+{
+    TileArgs a;
+    a.irec = irec;
+    a.jrec = jrec;
+    a.n_a = nA;
+    a.n_s = nB;
+    a.self_pass = self ? 1 : 0;
+    a.eps2 = c->eps2;
+    a.nsplit = tile_splits(nA, nB, c->n_sm, c->part_elems);
+    a.part = L.part;
+    return a;
+}
+
 // Newtonian accelerations of A from B (self: the same list); writes G * sum into out_soa
 // ([3][nA]) and, if given, out_aos ([nA][3]).  With wmax (mixed mode), also the weight
 // max_j m_j / r^3 of each particle's dominant term, which the following gradient pass uses.
 // With hist (mixed mode, with wmax): the |a| histogram of the pass is added to hist (zeroed by
 // the caller) for the hot-source classification of mark_hot.  kick: the kick of A by the
 // result, fused into the finalisation.  irec / jrec: records already packed by the caller
-// (NULL: packed here into the lane's recA / recB).
+// (NULL: packed here into the lane's recA / recB).  tile: the lists are in spatial order and
+// take the tile kernels (packed records are theirs); omap: the rows of out_aos.
 bool use_sym_self(const frost_ctx *c, int n) { return c->sym_cross > 0 || (c->sym_cross == 0 && n >= kSymTstepMinN); }
 
 void pass_acc(frost_ctx *c, Lane &L, const int32_t *A, int nA, const int32_t *B, int nB, bool self,
               double *out_soa, double *out_aos, float *wmax = nullptr, unsigned *hist = nullptr,
               KickArgs kick = KickArgs(), const void *irec = nullptr, const void *jrec = nullptr,
-              bool wmax_ready = false)
+              bool wmax_ready = false, bool tile = false, const int32_t *omap = nullptr)
 {
     if (nA <= 0) return;
     if (nB <= 0 || (self && nA == 1)) {
@@ -466,6 +489,28 @@ void pass_acc(frost_ctx *c, Lane &L, const int32_t *A, int nA, const int32_t *B,
     // same position records: a prepass for wmax = max_j m_j / r^3, then the pass with
     // Newton-refined rsqrt, short folds and the terms above wmax / 16 in double-float
     const bool accurate = c->mixed && wmax;
+    const int64_t pairs = self ? (int64_t)nA * (nA - 1) : (int64_t)nA * nB;
+    if (tile) {
+        if (!irec) {
+            launch_tile_pack_pos(L.s, A, nA, c->x, nullptr, 0.0, c->m, c->N, L.recA);
+            if (!self) launch_tile_pack_pos(L.s, B, nB, c->x, nullptr, 0.0, c->m, c->N, L.recB);
+            c->st.kernel_launches += self ? 1 : 2;
+        }
+        const TileArgs t = tile_args(c, L, irec ? irec : L.recA, nA, irec ? jrec : (self ? L.recA : L.recB), nB, self);
+        {
+            TimedScope ts(c, L.s, PASS_ACC, pairs);
+            if (accurate) launch_wmax_tile(L.s, t, c->n_sm, wmax);
+            launch_acc_tile(L.s, t, accurate ? wmax : nullptr);
+        }
+        launch_finalize_vec(L.s, L.part, t.nsplit, nA, c->G, out_soa, out_aos, &c->dmisc->err, badbit(c), kick, omap);
+        c->st.kernel_launches += accurate ? 3 : 2;
+        c->st.acc_pairs += pairs;
+        if (accurate && hist && out_soa) {
+            launch_acc_hist(L.s, out_soa, nA, hist);
+            c->st.kernel_launches += 1;
+        }
+        return;
+    }
     if (irec) {
         // packed by the caller
     } else {
@@ -485,7 +530,6 @@ void pass_acc(frost_ctx *c, Lane &L, const int32_t *A, int nA, const int32_t *B,
     a.wmax = accurate ? wmax : nullptr;
     a.jlist = B;
     a.m = c->m;
-    const int64_t pairs = self ? (int64_t)nA * (nA - 1) : (int64_t)nA * nB;
     {
         TimedScope ts(c, L.s, PASS_ACC, pairs);
         if (accurate && !wmax_ready) {
@@ -536,7 +580,8 @@ unsigned *zero_hists(Lane &L)
 void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA, const int32_t *B, int nB,
                const double *aB, bool self, double eps_grad, double *at_soa, double *at_aos,
                double *g_aos, const float *wmax, const uint32_t *hotB = nullptr,
-               KickArgs kick = KickArgs(), const void *irec = nullptr, const void *jrec = nullptr)
+               KickArgs kick = KickArgs(), const void *irec = nullptr, const void *jrec = nullptr, bool tile = false,
+               const int32_t *omap = nullptr)
 {
     if (nA <= 0) return;
     const double cgrad = eps_grad * eps_grad / 48.0;
@@ -551,6 +596,9 @@ void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA
     if (!c->mixed) hotB = nullptr;
     if (irec) {
         // packed by the caller
+    } else if (tile) {
+        launch_tile_pack_grad(L.s, A, nA, c->x, c->m, c->N, aA, self ? hotB : nullptr, L.recA);
+        if (!self) launch_tile_pack_grad(L.s, B, nB, c->x, c->m, c->N, aB, hotB, L.recB);
     } else if (c->mixed) {
         // hot sources: masses zeroed in the FP32 source records, their terms summed in
         // double-float by k_grad_hot
@@ -561,18 +609,26 @@ void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA
         if (!self) launch_pack_grad_fp64(L.s, B, nB, c->x, c->m, c->N, aB, (double4_32a *)L.recB);
     }
     if (!irec) c->st.kernel_launches += self ? 1 : 2;
-    PairArgs a;
-    a.irec = irec ? irec : L.recA;
-    a.jrec = irec ? jrec : (self ? L.recA : L.recB);
-    a.n_a = nA;
-    a.n_s = nB;
-    a.self_pass = self ? 1 : 0;
-    a.eps2 = c->eps2;
-    a.part = L.part;
-    a.shape = shape_for(c, PASS_GRAD, nA, nB);
-    a.wmax = c->mixed ? wmax : nullptr;
+    const void *ir = irec ? irec : L.recA, *jr = irec ? jrec : (self ? L.recA : L.recB);
     const int64_t pairs = self ? (int64_t)nA * (nA - 1) : (int64_t)nA * nB;
-    {
+    int nsplit;
+    if (tile) {
+        const TileArgs t = tile_args(c, L, ir, nA, jr, nB, self);
+        nsplit = t.nsplit;
+        TimedScope ts(c, L.s, PASS_GRAD, pairs);
+        launch_grad_tile(L.s, t, wmax);
+    } else {
+        PairArgs a;
+        a.irec = ir;
+        a.jrec = jr;
+        a.n_a = nA;
+        a.n_s = nB;
+        a.self_pass = self ? 1 : 0;
+        a.eps2 = c->eps2;
+        a.part = L.part;
+        a.shape = shape_for(c, PASS_GRAD, nA, nB);
+        a.wmax = c->mixed ? wmax : nullptr;
+        nsplit = a.shape.nsplit;
         TimedScope ts(c, L.s, PASS_GRAD, pairs);
         launch_grad(L.s, c->mixed, a);
     }
@@ -580,12 +636,12 @@ void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA
     if (hotB) {
         ns_hot = hot_grad_splits(nA, nB, c->n_sm);
         while (ns_hot > 1 && (size_t)ns_hot * 3 * nA > c->part_hot_elems) --ns_hot;
-        launch_grad_hot(L.s, A, nA, aA, B, nB, aB, hotB, a.self_pass, c->x, c->m, c->N, c->eps2, ns_hot,
+        launch_grad_hot(L.s, A, nA, aA, B, nB, aB, hotB, self ? 1 : 0, c->x, c->m, c->N, c->eps2, ns_hot,
                         L.part_hot);
         c->st.kernel_launches += 1;
     }
-    launch_finalize_grad(L.s, L.part, a.shape.nsplit, nA, 2.0 * c->G, aA, cgrad, at_soa, at_aos, g_aos,
-                         &c->dmisc->err, badbit(c), L.part_hot, ns_hot, kick);
+    launch_finalize_grad(L.s, L.part, nsplit, nA, 2.0 * c->G, aA, cgrad, at_soa, at_aos, g_aos, &c->dmisc->err, badbit(c),
+                         L.part_hot, ns_hot, kick, omap);
     c->st.kernel_launches += 2;
     c->st.grad_pairs += pairs;
 }
@@ -670,26 +726,38 @@ KickArgs kick_of(frost_ctx *c, const int32_t *list, double dt)
 }
 
 // drift of the list, writing the position records of the Newtonian pass that follows into rec
-void drift_pack(frost_ctx *c, Lane &L, const int32_t *list, int n, double dt, void *rec)
+void drift_pack(frost_ctx *c, Lane &L, const int32_t *list, int n, double dt, void *rec, bool tile)
 {
     if (n <= 0) return;
+    if (tile) {
+        launch_tile_pack_pos(L.s, list, n, c->x, c->v, dt, c->m, c->N, rec);
+        c->st.kernel_launches += 1;
+        return;
+    }
     launch_drift_pack(L.s, list, n, c->x, c->v, c->m, c->N, dt, rec, c->mixed ? 0 : 2);
     c->st.kernel_launches += 1;
 }
 
 // position records of the list for a Newtonian pass (both variants read the same records)
-void pack_acc(frost_ctx *c, Lane &L, const int32_t *list, int n, void *rec)
+void pack_acc(frost_ctx *c, Lane &L, const int32_t *list, int n, void *rec, bool tile = false)
 {
     if (n <= 0) return;
+    if (tile) {
+        launch_tile_pack_pos(L.s, list, n, c->x, nullptr, 0.0, c->m, c->N, rec);
+        c->st.kernel_launches += 1;
+        return;
+    }
     pack_pos(c, L, list, n, rec);
 }
 
 // gradient records of the list with accelerations a ([3][n]); mixed mode: masses of the hot
 // particles (mask) zeroed, their terms are summed in double-float by k_grad_hot
-void pack_grad(frost_ctx *c, Lane &L, const int32_t *list, int n, const double *a, void *rec, const uint32_t *mask)
+void pack_grad(frost_ctx *c, Lane &L, const int32_t *list, int n, const double *a, void *rec, const uint32_t *mask,
+               bool tile = false)
 {
     if (n <= 0) return;
-    if (c->mixed) launch_pack_grad_mixed(L.s, list, n, c->x, c->m, c->N, a, (float4 *)rec, mask);
+    if (tile) launch_tile_pack_grad(L.s, list, n, c->x, c->m, c->N, a, mask, rec);
+    else if (c->mixed) launch_pack_grad_mixed(L.s, list, n, c->x, c->m, c->N, a, (float4 *)rec, mask);
     else launch_pack_grad_fp64(L.s, list, n, c->x, c->m, c->N, a, (double4_32a *)rec);
     c->st.kernel_launches += 1;
 }
@@ -704,27 +772,29 @@ void fsi(frost_ctx *c, Lane &L, const int32_t *S, int nS, double dt, int cache =
     if (nS <= 0) return;
     c->st.fsi_calls += 1;
     if (nS < 2) cache = 0;
+    const bool tile = tile_force(c, nS, nS);
     if (cache == 2) {
         launch_kick_by_particle(L.s, S, nS, c->v, c->N, c->aC, dt / 6.0);
         c->st.kernel_launches += 1;
         c->st.acc_pairs_reused += (int64_t)nS * (nS - 1);
     } else {
-        pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, nullptr, nullptr, kick_of(c, S, dt / 6.0));
+        pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, nullptr, nullptr, kick_of(c, S, dt / 6.0), nullptr, nullptr,
+                 false, tile);
     }
-    drift_pack(c, L, S, nS, 0.5 * dt, L.recA);
+    drift_pack(c, L, S, nS, 0.5 * dt, L.recA, tile);
     if (c->mixed) {
         unsigned *h = zero_hists(L);
-        pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, L.wA, h, KickArgs(), L.recA, L.recA);
+        pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, L.wA, h, KickArgs(), L.recA, L.recA, false, tile);
         mark_hot(c, L, nS, nS, true, L.aA, h, nullptr, 0, L.hA);
     } else {
         pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, L.wA, nullptr, KickArgs(), L.recA, L.recA);
     }
     pass_grad(c, L, S, nS, L.aA, S, nS, L.aA, true, dt, L.atA, nullptr, nullptr, L.wA, L.hA,
-              kick_of(c, S, 2.0 * dt / 3.0));
-    drift_pack(c, L, S, nS, 0.5 * dt, L.recA);
+              kick_of(c, S, 2.0 * dt / 3.0), nullptr, nullptr, tile);
+    drift_pack(c, L, S, nS, 0.5 * dt, L.recA, tile);
     KickArgs last = kick_of(c, S, dt / 6.0);
     if (cache == 1) last.store = c->aC;
-    pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, nullptr, nullptr, last, L.recA, L.recA);
+    pass_acc(c, L, S, nS, S, nS, true, L.aA, nullptr, nullptr, nullptr, last, L.recA, L.recA, false, tile);
 }
 
 // Newtonian accelerations of two disjoint lists due to each other with every pair evaluated
@@ -890,23 +960,27 @@ void kick_sf(frost_ctx *c, Lane &M, Lane *Bl, const int32_t *S, int nS, const in
              bool gradient, double tau_pivot)
 {
     if (nS <= 0 || nF <= 0) return;
-    pack_acc(c, M, S, nS, M.recA);
-    pack_acc(c, M, F, nF, M.recB);
+    const bool tile = tile_force(c, nS, nF);
+    pack_acc(c, M, S, nS, M.recA, tile);
+    pack_acc(c, M, F, nF, M.recB, tile);
     Branch br(c, Bl ? Bl : &M, true);
     if (!Bl) br.concurrent = false;
     Lane &X = Bl ? br.exec : M;
     if (!gradient) {
         // each S x F pair once, when the symmetric grid fills the GPU
-        if (c->sym_cross >= 0 && pass_acc_sym(c, M, S, nS, F, nF, M.aA, M.aB, kick_of(c, S, cdt),
-                                              kick_of(c, F, cdt), M.recA, M.recB, c->sym_cross > 0))
+        if (!tile && c->sym_cross >= 0 &&
+            pass_acc_sym(c, M, S, nS, F, nF, M.aA, M.aB, kick_of(c, S, cdt), kick_of(c, F, cdt), M.recA, M.recB,
+                         c->sym_cross > 0))
             return;
         br.fork();
-        pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, nullptr, nullptr, kick_of(c, S, cdt), M.recA, M.recB);
-        pass_acc(c, X, F, nF, S, nS, false, M.aB, nullptr, nullptr, nullptr, kick_of(c, F, cdt), M.recB, M.recA);
+        pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, nullptr, nullptr, kick_of(c, S, cdt), M.recA, M.recB, false,
+                 tile);
+        pass_acc(c, X, F, nF, S, nS, false, M.aB, nullptr, nullptr, nullptr, kick_of(c, F, cdt), M.recB, M.recA, false,
+                 tile);
         return;  // joined by br
     }
     // each S x F pair once for both sides: always with sym_cross = 1, else for small lists
-    if (c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF <= kSymGradMaxPairs) &&
+    if (!tile && c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF <= kSymGradMaxPairs) &&
         grad_pairwise_sym(c, M, S, nS, F, nF, tau_pivot, M.atA, M.atB, nullptr, nullptr, nullptr, nullptr,
                           kick_of(c, S, cdt), kick_of(c, F, cdt), true))
         return;
@@ -914,28 +988,28 @@ void kick_sf(frost_ctx *c, Lane &M, Lane *Bl, const int32_t *S, int nS, const in
     // the prepasses of both accurate passes in one symmetric kernel (each pair once), where
     // the lists are large
     bool wready = false;
-    if (c->mixed && c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF >= kSymCrossPrepassMinPairs)) {
+    if (!tile && c->mixed && c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF >= kSymCrossPrepassMinPairs)) {
         TimedScope ts(c, M.s, PASS_ACC, 0);
         launch_wmax_sym_cross(M.s, M.recA, nS, M.recB, nF, c->eps2, c->n_sm, M.wA, M.wB);
         c->st.kernel_launches += 1;
         wready = true;
     }
     br.fork();
-    pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, M.wA, h, KickArgs(), M.recA, M.recB, wready);
+    pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, M.wA, h, KickArgs(), M.recA, M.recB, wready, tile);
     pass_acc(c, X, F, nF, S, nS, false, M.aB, nullptr, M.wB, h ? h + HOT_BINS : nullptr, KickArgs(), M.recB,
-             M.recA, wready);
+             M.recA, wready, tile);
     br.join();
     if (h) {
         mark_hot(c, M, nS, nF, false, M.aA, h, h + HOT_BINS, nF, M.hA);
         mark_hot(c, M, nF, nS, false, M.aB, h + HOT_BINS, h, nS, M.hB);
     }
-    pack_grad(c, M, S, nS, M.aA, M.recA, c->mixed ? M.hA : nullptr);
-    pack_grad(c, M, F, nF, M.aB, M.recB, c->mixed ? M.hB : nullptr);
+    pack_grad(c, M, S, nS, M.aA, M.recA, c->mixed ? M.hA : nullptr, tile);
+    pack_grad(c, M, F, nF, M.aB, M.recB, c->mixed ? M.hB : nullptr, tile);
     br.fork();
     pass_grad(c, M, S, nS, M.aA, F, nF, M.aB, false, tau_pivot, M.atA, nullptr, nullptr, M.wA, M.hB,
-              kick_of(c, S, cdt), M.recA, M.recB);
+              kick_of(c, S, cdt), M.recA, M.recB, tile);
     pass_grad(c, X, F, nF, M.aB, S, nS, M.aA, false, tau_pivot, M.atB, nullptr, nullptr, M.wB, M.hA,
-              kick_of(c, F, cdt), M.recB, M.recA);
+              kick_of(c, F, cdt), M.recB, M.recA, tile);
 }
 
 frost_status ensure_level(frost_ctx *c, int depth)
@@ -1481,11 +1555,21 @@ frost_status frost_accel_gradient(frost_ctx *c, const int32_t *active, int64_t n
     const bool want_grad = acc_tilde || grad;
     Lane &M = c->main;
     if (self) {
+        // a large set in spatial order, the results in the caller's
+        const bool tile = c->ord && nA >= kOrderForceMinN;
+        const int32_t *P = A, *omap = nullptr;
+        if (tile) {
+            order_list(c, active, nA, c->opos, c->olist);
+            P = c->olist;
+            omap = c->opos;
+        }
         unsigned *h = (want_grad && c->mixed) ? zero_hists(M) : nullptr;
-        pass_acc(c, M, A, nA, A, nA, true, c->aA, acc, want_grad ? c->wA : nullptr, h);
+        pass_acc(c, M, P, nA, P, nA, true, c->aA, acc, want_grad ? c->wA : nullptr, h, KickArgs(), nullptr, nullptr,
+                 false, tile, omap);
         if (h) mark_hot(c, M, nA, nA, true, c->aA, h, nullptr, 0, c->hA);
         if (want_grad)
-            pass_grad(c, M, A, nA, c->aA, A, nA, c->aA, true, eps_grad, nullptr, acc_tilde, grad, c->wA, c->hA);
+            pass_grad(c, M, P, nA, c->aA, P, nA, c->aA, true, eps_grad, nullptr, acc_tilde, grad, c->wA, c->hA,
+                      KickArgs(), nullptr, nullptr, tile, omap);
     } else if (want_grad && c->mixed && nB > 0 && c->sym_cross >= 0 &&
                (c->sym_cross > 0 || (int64_t)nA * nB >= kSymCrossPrepassMinPairs)) {
         // both accurate passes on records packed once, their prepasses in one symmetric kernel
@@ -1650,7 +1734,14 @@ frost_status frost_fsi(frost_ctx *c, const int32_t *set, int64_t n_set, double d
 {
     if (!c) return fail(FROST_EINVAL, "NULL context");
     FROST_TRY(check_sizes(c, n_set, "n_set"));
-    fsi(c, c->main, set ? set : c->all, (int)n_set, dt);
+    if (use_order(c, (int)n_set)) {
+        order_list(c, set, (int)n_set, c->opos, c->olist);
+        c->ordered = true;
+        fsi(c, c->main, c->olist, (int)n_set, dt);
+        c->ordered = false;
+    } else {
+        fsi(c, c->main, set ? set : c->all, (int)n_set, dt);
+    }
     FROST_CUDA(cudaGetLastError());
     return FROST_OK;
 }
@@ -1660,9 +1751,12 @@ void leapfrog(frost_ctx *c, const int32_t *S, int nS, double h)
 {
     if (nS <= 0) return;
     Lane &M = c->main;
-    pass_acc(c, M, S, nS, S, nS, true, c->aA, nullptr, nullptr, nullptr, kick_of(c, S, 0.5 * h));
-    drift_pack(c, M, S, nS, h, c->recA);
-    pass_acc(c, M, S, nS, S, nS, true, c->aA, nullptr, nullptr, nullptr, kick_of(c, S, 0.5 * h), c->recA, c->recA);
+    const bool tile = tile_force(c, nS, nS);
+    pass_acc(c, M, S, nS, S, nS, true, c->aA, nullptr, nullptr, nullptr, kick_of(c, S, 0.5 * h), nullptr, nullptr, false,
+             tile);
+    drift_pack(c, M, S, nS, h, c->recA, tile);
+    pass_acc(c, M, S, nS, S, nS, true, c->aA, nullptr, nullptr, nullptr, kick_of(c, S, 0.5 * h), c->recA, c->recA, false,
+             tile);
 }
 
 // The second-order HOLD integrator, Eq. hhs2: e^{eps/2 H_F} e^{eps/2 H_S} e^{eps U_FS}

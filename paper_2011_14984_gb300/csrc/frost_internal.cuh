@@ -123,16 +123,17 @@ struct KickArgs {
 };
 
 // out_soa[c][i] = scale * sum_split part[split][c][i]  (also [i][3] copy if out_aos != NULL),
-// then the kick / store of kick
+// then the kick / store of kick.  omap (optional): the row of out_aos that entry i goes to
 void launch_finalize_vec(cudaStream_t s, const double *part, int nsplit, int n, double scale,
                          double *out_soa, double *out_aos, int *err, int coincident_bit,
-                         KickArgs kick = KickArgs());
+                         KickArgs kick = KickArgs(), const int32_t *omap = nullptr);
 // a~ = a + c g with g = scale * (sum part + sum part2); writes a~ (soa and/or aos) and g
 // (aos, optional); part2 (nsplit2 splits, may be 0) holds the double-float terms of hot sources
 void launch_finalize_grad(cudaStream_t s, const double *part, int nsplit, int n, double scale,
                           const double *a_soa, double c, double *at_soa, double *at_aos,
                           double *g_aos, int *err, int coincident_bit,
-                          const double *part2 = nullptr, int nsplit2 = 0, KickArgs kick = KickArgs());
+                          const double *part2 = nullptr, int nsplit2 = 0, KickArgs kick = KickArgs(),
+                          const int32_t *omap = nullptr);
 
 // ---- hot sources of the mixed gradient pass (hot_kernels.cu) -------------------------
 constexpr int HOT_BINS = 1024;          // |a| histogram: 4 bins per octave
@@ -274,6 +275,32 @@ void launch_spatial_order(cudaStream_t s, const int32_t *list, int n, const doub
 void launch_tstep_tile(cudaStream_t s, const int32_t *list, int n, const double *x, const double *v, const double *m,
                        int N, double G, double eta, int sym, int n_sm, void *rec, unsigned *best, const int32_t *pos,
                        double *tau, int *err);
+
+// Mixed Newtonian and gradient passes of spatially ordered lists (force_tiles.cu).  rec: tiles of
+// TILE_N particles, TILE_POS_ROWS or TILE_GRAD_ROWS rows of TILE_N floats, then the tiles' heads.
+constexpr int TILE_N = 64;
+constexpr int TILE_POS_ROWS = 9, TILE_GRAD_ROWS = 13, TILE_HEAD_BYTES = 64;
+struct TileArgs {
+    const void *irec, *jrec;
+    int n_a, n_s;
+    int self_pass;   // 1 if the two lists are the same list
+    double eps2;     // softening^2
+    int nsplit;      // j-splits (tile_splits)
+    double *part;    // partial results [nsplit][3][n_a]
+};
+int tile_splits(int n_a, int n_s, int n_sm, size_t part_elems);
+// position records; v (optional): after a drift by dt v (x is then written)
+void launch_tile_pack_pos(cudaStream_t s, const int32_t *list, int n, double *x, const double *v, double dt,
+                          const double *m, int N, void *rec);
+// gradient records with accelerations acc ([3][n] by list position); hot (optional): mask of
+// the sources whose terms are summed elsewhere
+void launch_tile_pack_grad(cudaStream_t s, const int32_t *list, int n, const double *x, const double *m, int N,
+                           const double *acc, const uint32_t *hot, void *rec);
+// wmax[i] = max_j m_j / r^3 (zeroed here), for the Newtonian pass that feeds a gradient (wmax
+// given) and for the gradient; without wmax the plain Newtonian pass
+void launch_wmax_tile(cudaStream_t s, const TileArgs &a, int n_sm, float *wmax);
+void launch_acc_tile(cudaStream_t s, const TileArgs &a, const float *wmax);
+void launch_grad_tile(cudaStream_t s, const TileArgs &a, const float *wmax);
 
 // ---- single-CTA subtree solver (subtree.cu) ------------------------------------------
 constexpr int SUBTREE_MAX_FRAMES = 64;  // recursion frames per block (max_depth < 64)

@@ -257,18 +257,19 @@ __device__ __forceinline__ double split_sum(const double *__restrict__ q, int ns
 
 __global__ void k_finalize_vec(const double *__restrict__ part, int nsplit, int n, double scale,
                                double *__restrict__ out_soa, double *__restrict__ out_aos,
-                               int *__restrict__ err, int badbit, KickArgs kick)
+                               int *__restrict__ err, int badbit, KickArgs kick, const int32_t *__restrict__ omap)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     bool ok = true;
+    const int oi = omap ? omap[i] : i;
     const int gi = (kick.v || kick.store) ? (kick.list ? kick.list[i] : i) : 0;
     for (int c = 0; c < 3; ++c) {
         double s = split_sum(part + (size_t)c * n + i, nsplit, (size_t)3 * n);
         s *= scale;
         ok = ok && isfinite(s);
         if (out_soa) out_soa[(size_t)c * n + i] = s;
-        if (out_aos) out_aos[(size_t)i * 3 + c] = s;
+        if (out_aos) out_aos[(size_t)oi * 3 + c] = s;
         // the kick that follows the pass: the roundings of k_kick (no contraction)
         if (kick.v) kick.v[(size_t)c * kick.N + gi] = __dadd_rn(kick.v[(size_t)c * kick.N + gi], __dmul_rn(kick.dt, s));
         if (kick.store) kick.store[(size_t)c * kick.N + gi] = s;
@@ -280,11 +281,13 @@ __global__ void k_finalize_grad(const double *__restrict__ part, int nsplit, int
                                 const double *__restrict__ a_soa, double c,
                                 double *__restrict__ at_soa, double *__restrict__ at_aos,
                                 double *__restrict__ g_aos, int *__restrict__ err, int badbit,
-                                const double *__restrict__ part2, int nsplit2, KickArgs kick)
+                                const double *__restrict__ part2, int nsplit2, KickArgs kick,
+                                const int32_t *__restrict__ omap)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     bool ok = true;
+    const int oi = omap ? omap[i] : i;
     const int gi = kick.v ? (kick.list ? kick.list[i] : i) : 0;
     for (int k = 0; k < 3; ++k) {
         double s = split_sum(part + (size_t)k * n + i, nsplit, (size_t)3 * n);
@@ -293,8 +296,8 @@ __global__ void k_finalize_grad(const double *__restrict__ part, int nsplit, int
         const double at = a_soa[(size_t)k * n + i] + c * g;
         ok = ok && isfinite(at) && isfinite(g);
         if (at_soa) at_soa[(size_t)k * n + i] = at;
-        if (at_aos) at_aos[(size_t)i * 3 + k] = at;
-        if (g_aos) g_aos[(size_t)i * 3 + k] = g;
+        if (at_aos) at_aos[(size_t)oi * 3 + k] = at;
+        if (g_aos) g_aos[(size_t)oi * 3 + k] = g;
         if (kick.v) kick.v[(size_t)k * kick.N + gi] = __dadd_rn(kick.v[(size_t)k * kick.N + gi], __dmul_rn(kick.dt, at));
     }
     if (!ok) atomicOr(err, badbit);
@@ -525,20 +528,21 @@ void launch_tstep(cudaStream_t s, bool mixed, const PairArgs &a, double eta, int
 }
 
 void launch_finalize_vec(cudaStream_t s, const double *part, int nsplit, int n, double scale,
-                         double *out_soa, double *out_aos, int *err, int badbit, KickArgs kick)
+                         double *out_soa, double *out_aos, int *err, int badbit, KickArgs kick,
+                         const int32_t *omap)
 {
     if (n <= 0) return;
-    k_finalize_vec<<<cdiv(n, 256), 256, 0, s>>>(part, nsplit, n, scale, out_soa, out_aos, err, badbit, kick);
+    k_finalize_vec<<<cdiv(n, 256), 256, 0, s>>>(part, nsplit, n, scale, out_soa, out_aos, err, badbit, kick, omap);
 }
 
 void launch_finalize_grad(cudaStream_t s, const double *part, int nsplit, int n, double scale,
                           const double *a_soa, double c, double *at_soa, double *at_aos,
                           double *g_aos, int *err, int badbit, const double *part2, int nsplit2,
-                          KickArgs kick)
+                          KickArgs kick, const int32_t *omap)
 {
     if (n <= 0) return;
     k_finalize_grad<<<cdiv(n, 256), 256, 0, s>>>(part, nsplit, n, scale, a_soa, c, at_soa, at_aos,
-                                                  g_aos, err, badbit, part2, part2 ? nsplit2 : 0, kick);
+                                                  g_aos, err, badbit, part2, part2 ? nsplit2 : 0, kick, omap);
 }
 
 void launch_finalize_tau(cudaStream_t s, const double *part, int nsplit, int n, double eta,
