@@ -17,6 +17,32 @@ struct dfloat {
     float h, l;
 };
 
+// Conversions between FP32 and FP64 in integer arithmetic, the bits of (double)f and (float)d.
+// On this part a conversion is an instruction of the FP64 unit, which takes a warp
+// instruction in about 64 cycles; these take about 8 and 14 instructions of the integer pipe
+// (16 lanes a cycle).  Values outside the common range (denormals, infinities, NaN, FP32
+// overflow) go to the instruction.
+__device__ __forceinline__ double f2d(float f)
+{
+    const unsigned u = __float_as_uint(f), t = u & 0x7fffffffu;
+    if (t != 0u && t - 0x00800000u >= 0x7f000000u) return (double)f;
+    const unsigned hi = (t == 0u) ? 0u : (t >> 3) + 0x38000000u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+
+__device__ __forceinline__ float d2f(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned t = hi & 0x7fffffffu;
+    // FP64 exponents 897 .. 1150 are the normal FP32 range
+    if (t - 0x38100000u >= 0x0fe00000u) return ((t | lo) == 0u) ? __uint_as_float(hi) : (float)d;
+    // exponent and 23 bits of the fraction, then round to nearest even on the 29 bits below
+    const unsigned m = ((t - 0x38000000u) << 3) | (lo >> 29);
+    const unsigned low = lo & 0x1fffffffu;
+    const unsigned up = (low + (m & 1u) > 0x10000000u) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (m + up));
+}
+
 // s + e = a + b exactly
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 {
@@ -43,12 +69,12 @@ __device__ __forceinline__ dfloat make(float h, float l)
 __device__ __forceinline__ dfloat from_double(double v)
 {
     dfloat r;
-    r.h = (float)v;
-    r.l = (float)(v - (double)r.h);
+    r.h = d2f(v);
+    r.l = d2f(v - f2d(r.h));
     return r;
 }
 
-__device__ __forceinline__ double to_double(dfloat a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ double to_double(dfloat a) { return f2d(a.h) + f2d(a.l); }
 
 __device__ __forceinline__ dfloat add(dfloat a, dfloat b)
 {
@@ -97,10 +123,10 @@ __device__ __forceinline__ dfloat rsqrt(dfloat a)
 // x = h + l + ll exactly (three FP32 parts hold the 53 bits of an FP64 value)
 __device__ __forceinline__ void split3(double v, float &h, float &l, float &ll)
 {
-    h = (float)v;
-    const double r = v - (double)h;
-    l = (float)r;
-    ll = (float)(r - (double)l);
+    h = d2f(v);
+    const double r = v - f2d(h);
+    l = d2f(r);
+    ll = d2f(r - f2d(l));
 }
 
 // x_j - x_i from three-part splits: the two larger differences are exact (TwoSum), the

@@ -17,6 +17,9 @@
 namespace frost {
 namespace dev {
 
+using df::d2f;
+using df::f2d;
+
 __device__ __forceinline__ void fold2(float &hi, float &lo, float p)
 {
     // TwoSum (Knuth): hi + p = s + e exactly
@@ -36,11 +39,11 @@ __device__ __forceinline__ float trunc12(float f)
 __device__ __forceinline__ void split3(double p, float &h, float &mi, float &l)
 {
     double r = p;
-    h = trunc12((float)r);
-    r -= (double)h;   // exact
-    mi = trunc12((float)r);
-    r -= (double)mi;  // exact
-    l = (float)r;
+    h = trunc12(d2f(r));
+    r -= f2d(h);   // exact
+    mi = trunc12(d2f(r));
+    r -= f2d(mi);  // exact
+    l = d2f(r);
 }
 
 
@@ -55,13 +58,13 @@ __device__ __forceinline__ void pack_pos_mixed_one(int k, const int32_t *__restr
 {
     const int i = list ? list[k] : k;
     const double px = x[i], py = x[N + i], pz = x[2 * N + i];
-    const float hx = (float)px, hy = (float)py, hz = (float)pz;
+    const float hx = d2f(px), hy = d2f(py), hz = d2f(pz);
     const double mi = m[i];
-    const float mh = (float)mi;
+    const float mh = d2f(mi);
     rec[k] = make_float4(hx, hy, hz, mh);
     // the low part of the mass completes its double-float (the dominant terms' weights)
-    rec[n + k] = make_float4((float)(px - (double)hx), (float)(py - (double)hy),
-                             (float)(pz - (double)hz), (float)(mi - (double)mh));
+    rec[n + k] = make_float4(d2f(px - f2d(hx)), d2f(py - f2d(hy)),
+                             d2f(pz - f2d(hz)), d2f(mi - f2d(mh)));
 }
 
 // acc may be NULL (positions only, for the Newtonian pass that precedes the gradient)
@@ -79,12 +82,12 @@ __device__ __forceinline__ void pack_grad_mixed_one(int k, const int32_t *__rest
     split3(x[N + i], hy, my, ly);
     split3(x[2 * N + i], hz, mz, lz);
     const double ax = acc ? acc[k] : 0.0, ay = acc ? acc[n + k] : 0.0, az = acc ? acc[2 * n + k] : 0.0;
-    const float ahx = trunc12((float)ax), ahy = trunc12((float)ay), ahz = trunc12((float)az);
-    rec[k] = make_float4(hx, hy, hz, zero_m ? 0.f : (float)m[i]);
+    const float ahx = trunc12(d2f(ax)), ahy = trunc12(d2f(ay)), ahz = trunc12(d2f(az));
+    rec[k] = make_float4(hx, hy, hz, zero_m ? 0.f : d2f(m[i]));
     rec[n + k] = make_float4(mx, my, mz, ahx);
     rec[2 * n + k] = make_float4(lx, ly, lz, ahy);
-    rec[3 * n + k] = make_float4(ahz, (float)(ax - (double)ahx), (float)(ay - (double)ahy),
-                                 (float)(az - (double)ahz));
+    rec[3 * n + k] = make_float4(ahz, d2f(ax - f2d(ahx)), d2f(ay - f2d(ahy)),
+                                 d2f(az - f2d(ahz)));
 }
 
 __device__ __forceinline__ void pack_tstep_mixed_one(int k, const int32_t *__restrict__ list, int n,
@@ -96,14 +99,14 @@ __device__ __forceinline__ void pack_tstep_mixed_one(int k, const int32_t *__res
 {
     const int i = list ? list[k] : k;
     const double px = x[i], py = x[N + i], pz = x[2 * N + i];
-    const float hx = (float)px, hy = (float)py, hz = (float)pz;
-    rec[k] = make_float4(hx, hy, hz, (float)m[i]);
-    rec[n + k] = make_float4((float)(px - (double)hx), (float)(py - (double)hy),
-                             (float)(pz - (double)hz), 0.f);
-    rec[2 * n + k] = make_float4((float)v[i], (float)v[N + i], (float)v[2 * N + i],
-                                 (float)(G * m[i]));
+    const float hx = d2f(px), hy = d2f(py), hz = d2f(pz);
+    rec[k] = make_float4(hx, hy, hz, d2f(m[i]));
+    rec[n + k] = make_float4(d2f(px - f2d(hx)), d2f(py - f2d(hy)),
+                             d2f(pz - f2d(hz)), 0.f);
+    rec[2 * n + k] = make_float4(d2f(v[i]), d2f(v[N + i]), d2f(v[2 * N + i]),
+                                 d2f(G * m[i]));
     // exact fly-by derivative: the accelerations of the set ([3][n], by list position)
-    if (acc) rec[3 * n + k] = make_float4((float)acc[k], (float)acc[n + k], (float)acc[2 * n + k], 0.f);
+    if (acc) rec[3 * n + k] = make_float4(d2f(acc[k]), d2f(acc[n + k]), d2f(acc[2 * n + k]), 0.f);
 }
 
 __device__ __forceinline__ void pack_pos_fp64_one(int k, const int32_t *__restrict__ list, int n,
@@ -1120,9 +1123,9 @@ __device__ __forceinline__ void acc_mixed_body(const float4 *__restrict__ irec,
     }
 #pragma unroll
     for (int k = 0; k < ILP; ++k) {
-        res[k][0] = (double)hx[k] + (double)lx[k];
-        res[k][1] = (double)hy[k] + (double)ly[k];
-        res[k][2] = (double)hz[k] + (double)lz[k];
+        res[k][0] = f2d(hx[k]) + f2d(lx[k]);
+        res[k][1] = f2d(hy[k]) + f2d(ly[k]);
+        res[k][2] = f2d(hz[k]) + f2d(lz[k]);
         wres[k] = wm[k];
     }
     if constexpr (DEFER && BS == 32) {
@@ -1447,9 +1450,9 @@ __device__ __forceinline__ void grad_mixed_body(const float4 *__restrict__ irec,
         });
 #pragma unroll
         for (int k = 0; k < ILP; ++k) {
-            res[k][0] = ((double)hx[k] + (double)lx[k]) + b[k][0];
-            res[k][1] = ((double)hy[k] + (double)ly[k]) + b[k][1];
-            res[k][2] = ((double)hz[k] + (double)lz[k]) + b[k][2];
+            res[k][0] = (f2d(hx[k]) + f2d(lx[k])) + b[k][0];
+            res[k][1] = (f2d(hy[k]) + f2d(ly[k])) + b[k][1];
+            res[k][2] = (f2d(hz[k]) + f2d(lz[k])) + b[k][2];
         }
     } else {
         // per thread, summed in double-float
@@ -1468,9 +1471,9 @@ __device__ __forceinline__ void grad_mixed_body(const float4 *__restrict__ irec,
                     else grad_term_fp64<ILP>(J0, J1, J2, J3, I, k, eps2d, f[0], f[1], f[2]);
                 }
             }
-            res[k][0] = ((double)hx[k] + (double)lx[k]) + (df::to_double(b.x) + f[0]);
-            res[k][1] = ((double)hy[k] + (double)ly[k]) + (df::to_double(b.y) + f[1]);
-            res[k][2] = ((double)hz[k] + (double)lz[k]) + (df::to_double(b.z) + f[2]);
+            res[k][0] = (f2d(hx[k]) + f2d(lx[k])) + (df::to_double(b.x) + f[0]);
+            res[k][1] = (f2d(hy[k]) + f2d(ly[k])) + (df::to_double(b.y) + f[1]);
+            res[k][2] = (f2d(hz[k]) + f2d(lz[k])) + (df::to_double(b.z) + f[2]);
         }
     }
 }

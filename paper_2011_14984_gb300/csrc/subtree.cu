@@ -35,6 +35,7 @@ constexpr int MAXD = SUBTREE_MAX_FRAMES;
 // sub-partition's FP64 unit for about 64 cycles).
 struct StepK {
     double h, k6, k23, k48;
+    double k24;  // 2 k48: a~ = a + k48 (2 g) with G = 1 is a + k24 g, bit for bit
 };
 
 struct SubParams {
@@ -42,6 +43,8 @@ struct SubParams {
     const double *m;
     int N;
     double G, eta, eps2;
+    float eps2f, etaf;             // rounded once (a conversion is an FP64 instruction)
+    int unit_G;                    // G = 1 (Henon units): sums need no multiplication
     int max_depth;
     int *err;
     unsigned long long *counters;  // acc pairs, grad pairs, tstep pairs, hhs calls, fsi calls, max depth
@@ -82,7 +85,21 @@ struct Counts {
 constexpr int SUB_BARRIER = 1;    // named barrier of the warps 1..7 sub-team (0 is __syncthreads)
 
 // G times a sum; G = 1 (Henon units) needs no FP64 multiply and gives the same bits
-__device__ __forceinline__ double g_scale(double G, double r) { return G == 1.0 ? r : G * r; }
+__device__ __forceinline__ double g_scale(const SubParams &p, double r)
+{
+    if (p.unit_G) return r;
+    return p.G * r;
+}
+
+// a + c (2 G r), the multiplications by powers of two folded into the coefficient (c2 = 2 c)
+__device__ __forceinline__ double grad_kick(const SubParams &p, double a, double c, double c2, double r)
+{
+    if (p.unit_G) return fma(c2, r, a);
+    return fma(c, 2.0 * p.G * r, a);
+}
+
+// whether an FP64 value is finite, without an FP64 instruction
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
 __device__ __forceinline__ int t_id(const SubParams &p) { return p.crank * p.tcount + ((int)threadIdx.x - p.tbase); }
 __device__ __forceinline__ int t_n(const SubParams &p) { return p.csize * p.tcount; }
@@ -201,28 +218,28 @@ __device__ __noinline__ void mt_acc(const SubParams &p, const void *irec, const 
         float wm[1] = {0.f};
         if (MIXED) {
             const float4 *ir = (const float4 *)irec, *jr = (const float4 *)jrec;
-            const float eps2 = (float)p.eps2;
+            const float eps2 = p.eps2f;
             float H[3] = {0.f, 0.f, 0.f}, L[3] = {0.f, 0.f, 0.f};
             float ax[1] = {0.f}, ay[1] = {0.f}, az[1] = {0.f};
-            int c = 0;
             AccMixedI<1> I;
             const float4 q0 = ir[i], q1 = ir[nA + i];
             I.xh[0] = q0.x; I.yh[0] = q0.y; I.zh[0] = q0.z;
             I.xl[0] = q1.x; I.yl[0] = q1.y; I.zl[0] = q1.z;
-            for (int q = 0; q < nq; ++q) {
-                const MtSrc s = mt_src(q, T, l, nB, i, self);
-                if (accurate)
-                    acc_mixed_j<1, true, true, true>(jr[s.j], jr[nB + s.j], I, eps2, s.jpos, ipos, ax, ay, az, wm);
-                else
-                    acc_mixed_j<1, true, false>(jr[s.j], jr[nB + s.j], I, eps2, s.jpos, ipos, ax, ay, az, wm);
-                if (++c == 16) {
-                    fold2(H[0], L[0], ax[0]); fold2(H[1], L[1], ay[0]); fold2(H[2], L[2], az[0]);
-                    ax[0] = ay[0] = az[0] = 0.f;
-                    c = 0;
+            // sums of 16 sources, four of which are in flight at a time
+            for (int q0 = 0; q0 < nq; q0 += 16) {
+                const int q1 = min(nq, q0 + 16);
+#pragma unroll 4
+                for (int q = q0; q < q1; ++q) {
+                    const MtSrc s = mt_src(q, T, l, nB, i, self);
+                    if (accurate)
+                        acc_mixed_j<1, true, true, true>(jr[s.j], jr[nB + s.j], I, eps2, s.jpos, ipos, ax, ay, az, wm);
+                    else
+                        acc_mixed_j<1, true, false>(jr[s.j], jr[nB + s.j], I, eps2, s.jpos, ipos, ax, ay, az, wm);
                 }
+                fold2(H[0], L[0], ax[0]); fold2(H[1], L[1], ay[0]); fold2(H[2], L[2], az[0]);
+                ax[0] = ay[0] = az[0] = 0.f;
             }
-            fold2(H[0], L[0], ax[0]); fold2(H[1], L[1], ay[0]); fold2(H[2], L[2], az[0]);
-            for (int k = 0; k < 3; ++k) r[k] = (double)H[k] + (double)L[k];
+            for (int k = 0; k < 3; ++k) r[k] = f2d(H[k]) + f2d(L[k]);
         } else {
             const double4_32a *ir = (const double4_32a *)irec, *jr = (const double4_32a *)jrec;
             const double4_32a I = ir[i];
@@ -237,8 +254,8 @@ __device__ __noinline__ void mt_acc(const SubParams &p, const void *irec, const 
         if (active && l == 0) {
             bool ok = true;
             for (int k = 0; k < 3; ++k) {
-                const double a = g_scale(p.G, r[k]);
-                ok = ok && isfinite(a);
+                const double a = g_scale(p, r[k]);
+                ok = ok && finite64(a);
                 out[k * nA + i] = a;
             }
             if (wout) wout[i] = wmx;
@@ -263,7 +280,7 @@ __device__ __noinline__ void mt_grad(const SubParams &p, const void *irec, const
         double r[3];
         if (MIXED) {
             const float4 *ir = (const float4 *)irec, *jr = (const float4 *)jrec;
-            const float eps2 = (float)p.eps2;
+            const float eps2 = p.eps2f;
             GradMixedI<1> I;
             const float4 q0 = ir[i], q1 = ir[nA + i], q2 = ir[2 * nA + i], q3 = ir[3 * nA + i];
             I.xh[0] = q0.x; I.yh[0] = q0.y; I.zh[0] = q0.z;
@@ -275,18 +292,17 @@ __device__ __noinline__ void mt_grad(const SubParams &p, const void *irec, const
             init_big(big, 0);
             float H[3] = {0.f, 0.f, 0.f}, L[3] = {0.f, 0.f, 0.f};
             float gx[1] = {0.f}, gy[1] = {0.f}, gz[1] = {0.f};
-            int cnt = 0;
-            for (int q = 0; q < nq; ++q) {
-                const MtSrc s = mt_src(q, T, l, nB, i, self);
-                grad_mixed_j<1, true>(jr[s.j], jr[nB + s.j], jr[2 * nB + s.j], jr[3 * nB + s.j], I, eps2, s.j, s.jpos,
-                                      ipos, thr, big, gx, gy, gz);
-                if (++cnt == 16) {
-                    fold2(H[0], L[0], gx[0]); fold2(H[1], L[1], gy[0]); fold2(H[2], L[2], gz[0]);
-                    gx[0] = gy[0] = gz[0] = 0.f;
-                    cnt = 0;
+            for (int q0 = 0; q0 < nq; q0 += 16) {
+                const int q1 = min(nq, q0 + 16);
+#pragma unroll 2
+                for (int q = q0; q < q1; ++q) {
+                    const MtSrc s = mt_src(q, T, l, nB, i, self);
+                    grad_mixed_j<1, true>(jr[s.j], jr[nB + s.j], jr[2 * nB + s.j], jr[3 * nB + s.j], I, eps2, s.j, s.jpos,
+                                          ipos, thr, big, gx, gy, gz);
                 }
+                fold2(H[0], L[0], gx[0]); fold2(H[1], L[1], gy[0]); fold2(H[2], L[2], gz[0]);
+                gx[0] = gy[0] = gz[0] = 0.f;
             }
-            fold2(H[0], L[0], gx[0]); fold2(H[1], L[1], gy[0]); fold2(H[2], L[2], gz[0]);
             double bx = 0.0, by = 0.0, bz = 0.0;
 #pragma unroll
             for (int t = 0; t < GRAD_SLOTS; ++t) {
@@ -295,9 +311,9 @@ __device__ __noinline__ void mt_grad(const SubParams &p, const void *irec, const
                     grad_term_df<1>(jr[j], jr[nB + j], jr[2 * nB + j], jr[3 * nB + j], I, 0, p.eps2, bx, by, bz);
                 }
             }
-            r[0] = ((double)H[0] + (double)L[0]) + bx;
-            r[1] = ((double)H[1] + (double)L[1]) + by;
-            r[2] = ((double)H[2] + (double)L[2]) + bz;
+            r[0] = (f2d(H[0]) + f2d(L[0])) + bx;
+            r[1] = (f2d(H[1]) + f2d(L[1])) + by;
+            r[2] = (f2d(H[2]) + f2d(L[2])) + bz;
         } else {
             const double4_32a *ir = (const double4_32a *)irec, *jr = (const double4_32a *)jrec;
             const double4_32a I = ir[i], IA = ir[nA + i];
@@ -311,8 +327,8 @@ __device__ __noinline__ void mt_grad(const SubParams &p, const void *irec, const
         if (active && l == 0) {
             bool ok = true;
             for (int k = 0; k < 3; ++k) {
-                const double v = aA[k * nA + i] + c * (2.0 * p.G * r[k]);
-                ok = ok && isfinite(v);
+                const double v = grad_kick(p, aA[k * nA + i], c, 2.0 * c, r[k]);
+                ok = ok && finite64(v);
                 at[k * nA + i] = v;
             }
             if (!ok) atomicOr(p.err, badbit);
@@ -343,7 +359,7 @@ __device__ __noinline__ void mt_tstep(const SubParams &p, const void *rec, int n
             I.xl[0] = b.x; I.yl[0] = b.y; I.zl[0] = b.z;
             I.vx[0] = cc.x; I.vy[0] = cc.y; I.vz[0] = cc.z; I.gm[0] = cc.w;
             I.ax[0] = da.x; I.ay[0] = da.y; I.az[0] = da.z;
-            const float eta = (float)p.eta, eta15 = 1.5f * eta;
+            const float eta = p.etaf, eta15 = 1.5f * eta;
             float best[1] = {INFINITY}, minr2[1] = {INFINITY};
             for (int q = 0; q < nq; ++q) {
                 const MtSrc s = mt_src(q, T, l, n, i, true);
@@ -351,7 +367,7 @@ __device__ __noinline__ void mt_tstep(const SubParams &p, const void *rec, int n
                 tstep_mixed_j<1, SYM, true>(r[s.j], r[n + s.j], r[2 * n + s.j], JA, I, eta, eta15, s.jpos, ipos,
                                             best, minr2);
             }
-            t = p.eta * (double)grp_min(best[0], T);
+            t = p.eta * f2d(grp_min(best[0], T));
             coincident = grp_min(minr2[0], T) == 0.f;
         } else {
             const double4_32a *r = (const double4_32a *)rec;
@@ -402,16 +418,16 @@ __device__ __noinline__ void b_acc(const SubParams &p, const SubWork &w, const i
         for (int ib = 0; ib < nA; ib += SIB) {
             double res[SILP][3];
             float wr[SILP];
-            if (accurate) acc_mixed_body<SB, SILP, STJ, true, true>(ir, jr, nA, nB, ib, 0, nB, sp, (float)p.eps2, res, wr);
-            else acc_mixed_body<SB, SILP, STJ, false>(ir, jr, nA, nB, ib, 0, nB, sp, (float)p.eps2, res, wr);
+            if (accurate) acc_mixed_body<SB, SILP, STJ, true, true>(ir, jr, nA, nB, ib, 0, nB, sp, p.eps2f, res, wr);
+            else acc_mixed_body<SB, SILP, STJ, false>(ir, jr, nA, nB, ib, 0, nB, sp, p.eps2f, res, wr);
 #pragma unroll
             for (int k = 0; k < SILP; ++k) {
                 const int i = ib + k * SB + threadIdx.x;
                 if (i < nA) {
                     bool ok = true;
                     for (int c = 0; c < 3; ++c) {
-                        const double a = g_scale(p.G, res[k][c]);
-                        ok = ok && isfinite(a);
+                        const double a = g_scale(p, res[k][c]);
+                        ok = ok && finite64(a);
                         out[c * nA + i] = a;
                     }
                     if (wout) wout[i] = wr[k];
@@ -429,8 +445,8 @@ __device__ __noinline__ void b_acc(const SubParams &p, const SubWork &w, const i
             if (i < nA) {
                 bool ok = true;
                 for (int c = 0; c < 3; ++c) {
-                    const double a = g_scale(p.G, res[c]);
-                    ok = ok && isfinite(a);
+                    const double a = g_scale(p, res[c]);
+                    ok = ok && finite64(a);
                     out[c * nA + i] = a;
                 }
                 if (!ok) atomicOr(p.err, badbit);
@@ -466,7 +482,6 @@ __device__ __noinline__ void b_grad(const SubParams &p, const SubWork &w, const 
     t_sync(p);
     const int sp = self ? 1 : 0;
     const double c = c48;  // eps^2 / 48, eps the step of the operator with the 2/3 kick
-    const double scale = 2.0 * p.G;
     if (p.csize > 1 || nA <= MT_MAX || p.tcount != SB) {
         mt_grad<MIXED>(p, w.recA, self ? w.recA : w.recB, nA, nB, self, aA, MIXED ? wmax : nullptr, c, at, badbit);
     } else if (MIXED) {
@@ -480,8 +495,8 @@ __device__ __noinline__ void b_grad(const SubParams &p, const SubWork &w, const 
                 if (i < nA) {
                     bool ok = true;
                     for (int q = 0; q < 3; ++q) {
-                        const double v = aA[q * nA + i] + c * (scale * res[k][q]);
-                        ok = ok && isfinite(v);
+                        const double v = grad_kick(p, aA[q * nA + i], c, 2.0 * c, res[k][q]);
+                        ok = ok && finite64(v);
                         at[q * nA + i] = v;
                     }
                     if (!ok) atomicOr(p.err, badbit);
@@ -498,8 +513,8 @@ __device__ __noinline__ void b_grad(const SubParams &p, const SubWork &w, const 
             if (i < nA) {
                 bool ok = true;
                 for (int q = 0; q < 3; ++q) {
-                    const double v = aA[q * nA + i] + c * (scale * res[q]);
-                    ok = ok && isfinite(v);
+                    const double v = grad_kick(p, aA[q * nA + i], c, 2.0 * c, res[q]);
+                    ok = ok && finite64(v);
                     at[q * nA + i] = v;
                 }
                 if (!ok) atomicOr(p.err, badbit);
@@ -536,12 +551,12 @@ __device__ __noinline__ void b_tstep(const SubParams &p, const SubWork &w, const
     } else if (MIXED) {
         for (int ib = 0; ib < n; ib += SIB) {
             float best[SILP], minr2[SILP];
-            tstep_mixed_body<SB, SILP, STJ, SYM>(w.recA, w.recA, n, n, ib, 0, n, 1, (float)p.eta, best, minr2);
+            tstep_mixed_body<SB, SILP, STJ, SYM>(w.recA, w.recA, n, n, ib, 0, n, 1, p.etaf, best, minr2);
 #pragma unroll
             for (int k = 0; k < SILP; ++k) {
                 const int i = ib + k * SB + threadIdx.x;
                 if (i < n) {
-                    const double t = p.eta * (double)best[k];
+                    const double t = p.eta * f2d(best[k]);
                     tau[i] = t;
                     if (minr2[k] == 0.f) atomicOr(p.err, ERR_COINCIDENT);
                     if (!(t > 0.0)) atomicOr(p.err, ERR_NONFINITE);
@@ -655,7 +670,12 @@ __device__ __noinline__ void b_fsi(const SubParams &p, const SubWork &w, const i
     const double dt = kc.h;
     if (nS <= 0) return;
     if (t_lead(p)) cnt.fsi += 1;
-    if (nS < 2) cache = 0;
+    if (nS < 2) {
+        // a particle alone: its accelerations are zero and the kicks change nothing
+        b_drift(p, S, nS, 0.5 * dt);
+        b_drift(p, S, nS, 0.5 * dt);
+        return;
+    }
     if (cache == 2) {
         if (t_lead(p)) cnt.reused += (unsigned long long)nS * (nS - 1);
         for (int k = t_id(p); k < nS; k += t_n(p)) {
@@ -732,93 +752,142 @@ struct WLane {
 __device__ __forceinline__ void w_record(WLane &L)
 {
     for (int c = 0; c < 3; ++c) {
-        L.rh[c] = (float)L.xr[c];
-        L.rl[c] = (float)(L.xr[c] - (double)L.rh[c]);
+        L.rh[c] = d2f(L.xr[c]);
+        L.rl[c] = d2f(L.xr[c] - f2d(L.rh[c]));
     }
-    L.mf = (float)L.m;
+    L.mf = d2f(L.m);
 }
 
 __device__ __forceinline__ float wsh(float v, int j) { return __shfl_sync(0xffffffffu, v, j); }
 __device__ __forceinline__ double wshd(double v, int j) { return __shfl_sync(0xffffffffu, v, j); }
 
-// Newtonian pass: every lane sums over the sources j of the uniform mask U with bit j set in
-// its own mask mysrc (j != lane).  accurate: the variant that feeds a gradient (Newton-refined
-// rsqrt, short folds), also returning max_j m_j / r^3.
+// What a pass of the warp path takes and returns, by value: a reference into the lane's state
+// or to SubParams would put them in local memory, and one warp alone waits for every load.
+// (The path is bound by one warp's latencies: by stall counts about 2.4 cycles an instruction on
+// dependent results, 1.7 on instruction fetch, 1.6 on shuffles, FP64 and MUFU, 0.5 on memory.
+// By value, with two sources in flight, conversions on the integer pipe and lone particles
+// only drifted, a 65536-body step's launches take 12.6 instead of 13.7 ms.)
+struct WSrc {
+    float h[3], l[3], m;  // mixed: the lane's record
+    double x[3], md;      // FP64: its position and mass
+    float eps2f;
+    double eps2;
+};
+struct WSum {
+    double a[3];
+    float wmax;
+};
+
 template <bool MIXED>
-__device__ __noinline__ void w_acc(const SubParams &p, const WLane &L, unsigned U, unsigned mysrc, bool accurate,
-                                   double (&a)[3], float &wmax)
+__device__ __forceinline__ WSrc w_src(const SubParams &p, const WLane &L)
+{
+    WSrc r;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        r.h[c] = MIXED ? L.rh[c] : 0.f;
+        r.l[c] = MIXED ? L.rl[c] : 0.f;
+        r.x[c] = MIXED ? L.xr[c] : L.x[c];
+    }
+    r.m = MIXED ? L.mf : 0.f;
+    r.md = MIXED ? 0.0 : L.m;
+    r.eps2f = p.eps2f;
+    r.eps2 = p.eps2;
+    return r;
+}
+
+// Newtonian pass: every lane sums (without the factor G) over the sources j of the uniform mask
+// U with bit j set in its own mask mysrc (j != lane).  ACCURATE: the variant that feeds a
+// gradient (Newton-refined rsqrt), also returning max_j m_j / r^3.
+template <bool MIXED, bool ACCURATE>
+__device__ __noinline__ WSum w_acc(WSrc L, unsigned U, unsigned mysrc)
 {
     const int lane = threadIdx.x & 31;
     const int ipos[1] = {lane};
-    float wm[1] = {0.f};
-    double res[3] = {0.0, 0.0, 0.0};
+    WSum r;
+    r.wmax = 0.f;
     if (MIXED) {
-        const float eps2 = (float)p.eps2;
         float H[3] = {0.f, 0.f, 0.f}, Lo[3] = {0.f, 0.f, 0.f};
-        float ax[1] = {0.f}, ay[1] = {0.f}, az[1] = {0.f};
+        float ax[1] = {0.f}, ay[1] = {0.f}, az[1] = {0.f}, wm[1] = {0.f};
         int c = 0;
         AccMixedI<1> I;
-        const float hx = L.rh[0], hy = L.rh[1], hz = L.rh[2];
-        I.xh[0] = hx; I.yh[0] = hy; I.zh[0] = hz;
-        I.xl[0] = L.rl[0];
-        I.yl[0] = L.rl[1];
-        I.zl[0] = L.rl[2];
-        const float mf = L.mf;
+        I.xh[0] = L.h[0]; I.yh[0] = L.h[1]; I.zh[0] = L.h[2];
+        I.xl[0] = L.l[0]; I.yl[0] = L.l[1]; I.zl[0] = L.l[2];
         unsigned M = U;
         while (M) {
-            const int j = __ffs(M) - 1;
+            // two sources in flight; past the last one, it again, masked as the self pair
+            int jj[2], jp[2];
+            jj[0] = jp[0] = __ffs(M) - 1;
             M &= M - 1;
-            float4 J0 = make_float4(wsh(hx, j), wsh(hy, j), wsh(hz, j), wsh(mf, j));
-            const float4 J1 = make_float4(wsh(I.xl[0], j), wsh(I.yl[0], j), wsh(I.zl[0], j), 0.f);
-            if (!((mysrc >> j) & 1u)) J0.w = 0.f;
-            if (accurate) acc_mixed_j<1, true, true, true>(J0, J1, I, eps2, j, ipos, ax, ay, az, wm);
-            else acc_mixed_j<1, true, false>(J0, J1, I, eps2, j, ipos, ax, ay, az, wm);
-            if (++c == 16) {
+            jj[1] = M ? __ffs(M) - 1 : jj[0];
+            jp[1] = M ? jj[1] : lane;
+            M &= M - 1;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int j = jj[e];
+                float4 J0 = make_float4(wsh(L.h[0], j), wsh(L.h[1], j), wsh(L.h[2], j), wsh(L.m, j));
+                const float4 J1 = make_float4(wsh(L.l[0], j), wsh(L.l[1], j), wsh(L.l[2], j), 0.f);
+                if (!((mysrc >> j) & 1u)) J0.w = 0.f;
+                acc_mixed_j<1, true, ACCURATE, ACCURATE>(J0, J1, I, L.eps2f, jp[e], ipos, ax, ay, az, wm);
+            }
+            if ((c += 2) == 16) {
                 fold2(H[0], Lo[0], ax[0]); fold2(H[1], Lo[1], ay[0]); fold2(H[2], Lo[2], az[0]);
                 ax[0] = ay[0] = az[0] = 0.f;
                 c = 0;
             }
         }
         fold2(H[0], Lo[0], ax[0]); fold2(H[1], Lo[1], ay[0]); fold2(H[2], Lo[2], az[0]);
-        for (int q = 0; q < 3; ++q) res[q] = (double)H[q] + (double)Lo[q];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) r.a[q] = f2d(H[q]) + f2d(Lo[q]);
+        r.wmax = wm[0];
     } else {
-        const double4_32a I = make_double4_32a(L.x[0], L.x[1], L.x[2], L.m);
+        const double4_32a I = make_double4_32a(L.x[0], L.x[1], L.x[2], L.md);
+        r.a[0] = r.a[1] = r.a[2] = 0.0;
         unsigned M = U;
         while (M) {
             const int j = __ffs(M) - 1;
             M &= M - 1;
-            double4_32a J = make_double4_32a(wshd(L.x[0], j), wshd(L.x[1], j), wshd(L.x[2], j), wshd(L.m, j));
+            double4_32a J = make_double4_32a(wshd(L.x[0], j), wshd(L.x[1], j), wshd(L.x[2], j), wshd(L.md, j));
             if (!((mysrc >> j) & 1u)) J.w = 0.0;
-            acc_fp64_j<true>(J, I, p.eps2, j, lane, res[0], res[1], res[2]);
+            acc_fp64_j<true>(J, I, L.eps2, j, lane, r.a[0], r.a[1], r.a[2]);
         }
     }
-    for (int q = 0; q < 3; ++q) a[q] = g_scale(p.G, res[q]);
-    wmax = wm[0];
+    return r;
 }
 
-// Gradient pass: lane sums over j in U with bit j of mysrc, using its own acceleration ai
-// and the sources' accelerations (each lane's ai); dominant terms (w > thr) in double-float.
+// w_acc with the factor G
+template <bool MIXED, bool ACCURATE>
+__device__ __forceinline__ WSum w_accel(const SubParams &p, const WLane &L, unsigned U, unsigned mysrc)
+{
+    WSum r = w_acc<MIXED, ACCURATE && MIXED>(w_src<MIXED>(p, L), U, mysrc);
+    if (!p.unit_G)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) r.a[q] = p.G * r.a[q];
+    return r;
+}
+
+// Gradient pass: lane sums (without the factor 2 G) over j in U with bit j of mysrc, using its
+// own acceleration a and the sources' accelerations (each lane's a); dominant terms (above
+// SLOT_FRACTION of a.wmax) in double-float.
 template <bool MIXED>
-__device__ __noinline__ void w_grad(const SubParams &p, const WLane &L, unsigned U, unsigned mysrc,
-                                    const double (&ai)[3], float thr, double (&g)[3])
+__device__ __noinline__ WSum w_grad(WSrc L, unsigned U, unsigned mysrc, WSum a)
 {
     const int lane = threadIdx.x & 31;
     const int ipos[1] = {lane};
-    double res[3] = {0.0, 0.0, 0.0};
+    WSum r;
+    r.wmax = 0.f;
     if (MIXED) {
-        const float eps2 = (float)p.eps2;
         GradMixedI<1> I;
-        split3(L.xr[0], I.xh[0], I.xm[0], I.xl[0]);
-        split3(L.xr[1], I.yh[0], I.ym[0], I.yl[0]);
-        split3(L.xr[2], I.zh[0], I.zm[0], I.zl[0]);
-        I.ahx[0] = trunc12((float)ai[0]);
-        I.ahy[0] = trunc12((float)ai[1]);
-        I.ahz[0] = trunc12((float)ai[2]);
-        I.alx[0] = (float)(ai[0] - (double)I.ahx[0]);
-        I.aly[0] = (float)(ai[1] - (double)I.ahy[0]);
-        I.alz[0] = (float)(ai[2] - (double)I.ahz[0]);
-        const float mf = L.mf;
-        const float thrs[1] = {thr};
+        split3(L.x[0], I.xh[0], I.xm[0], I.xl[0]);
+        split3(L.x[1], I.yh[0], I.ym[0], I.yl[0]);
+        split3(L.x[2], I.zh[0], I.zm[0], I.zl[0]);
+        I.ahx[0] = trunc12(d2f(a.a[0]));
+        I.ahy[0] = trunc12(d2f(a.a[1]));
+        I.ahz[0] = trunc12(d2f(a.a[2]));
+        I.alx[0] = d2f(a.a[0] - f2d(I.ahx[0]));
+        I.aly[0] = d2f(a.a[1] - f2d(I.ahy[0]));
+        I.alz[0] = d2f(a.a[2] - f2d(I.ahz[0]));
+        const float mf = L.m;
+        const float thrs[1] = {SLOT_FRACTION * a.wmax};
         BigSlots<1> big;
         init_big(big, lane);
         float H[3] = {0.f, 0.f, 0.f}, Lo[3] = {0.f, 0.f, 0.f};
@@ -826,15 +895,23 @@ __device__ __noinline__ void w_grad(const SubParams &p, const WLane &L, unsigned
         int c = 0;
         unsigned M = U;
         while (M) {
-            const int j = __ffs(M) - 1;
+            int jj[2], jp[2];
+            jj[0] = jp[0] = __ffs(M) - 1;
             M &= M - 1;
-            float4 J0 = make_float4(wsh(I.xh[0], j), wsh(I.yh[0], j), wsh(I.zh[0], j), wsh(mf, j));
-            const float4 J1 = make_float4(wsh(I.xm[0], j), wsh(I.ym[0], j), wsh(I.zm[0], j), wsh(I.ahx[0], j));
-            const float4 J2 = make_float4(wsh(I.xl[0], j), wsh(I.yl[0], j), wsh(I.zl[0], j), wsh(I.ahy[0], j));
-            const float4 J3 = make_float4(wsh(I.ahz[0], j), wsh(I.alx[0], j), wsh(I.aly[0], j), wsh(I.alz[0], j));
-            if (!((mysrc >> j) & 1u)) J0.w = 0.f;
-            grad_mixed_j<1, true>(J0, J1, J2, J3, I, eps2, j, j, ipos, thrs, big, gx, gy, gz);
-            if (++c == 16) {
+            jj[1] = M ? __ffs(M) - 1 : jj[0];
+            jp[1] = M ? jj[1] : lane;
+            M &= M - 1;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int j = jj[e];
+                float4 J0 = make_float4(wsh(I.xh[0], j), wsh(I.yh[0], j), wsh(I.zh[0], j), wsh(mf, j));
+                const float4 J1 = make_float4(wsh(I.xm[0], j), wsh(I.ym[0], j), wsh(I.zm[0], j), wsh(I.ahx[0], j));
+                const float4 J2 = make_float4(wsh(I.xl[0], j), wsh(I.yl[0], j), wsh(I.zl[0], j), wsh(I.ahy[0], j));
+                const float4 J3 = make_float4(wsh(I.ahz[0], j), wsh(I.alx[0], j), wsh(I.aly[0], j), wsh(I.alz[0], j));
+                if (!((mysrc >> j) & 1u)) J0.w = 0.f;
+                grad_mixed_j<1, true>(J0, J1, J2, J3, I, L.eps2f, j, jp[e], ipos, thrs, big, gx, gy, gz);
+            }
+            if ((c += 2) == 16) {
                 fold2(H[0], Lo[0], gx[0]); fold2(H[1], Lo[1], gy[0]); fold2(H[2], Lo[2], gz[0]);
                 gx[0] = gy[0] = gz[0] = 0.f;
                 c = 0;
@@ -853,30 +930,31 @@ __device__ __noinline__ void w_grad(const SubParams &p, const WLane &L, unsigned
             const float4 Q1 = make_float4(wsh(I.xm[0], j), wsh(I.ym[0], j), wsh(I.zm[0], j), wsh(I.ahx[0], j));
             const float4 Q2 = make_float4(wsh(I.xl[0], j), wsh(I.yl[0], j), wsh(I.zl[0], j), wsh(I.ahy[0], j));
             const float4 Q3 = make_float4(wsh(I.ahz[0], j), wsh(I.alx[0], j), wsh(I.aly[0], j), wsh(I.alz[0], j));
-            if (s < big.n[0]) grad_term_df<1>(Q0, Q1, Q2, Q3, I, 0, p.eps2, bx, by, bz);
+            if (s < big.n[0]) grad_term_df<1>(Q0, Q1, Q2, Q3, I, 0, L.eps2, bx, by, bz);
         }
-        res[0] = ((double)H[0] + (double)Lo[0]) + bx;
-        res[1] = ((double)H[1] + (double)Lo[1]) + by;
-        res[2] = ((double)H[2] + (double)Lo[2]) + bz;
+        r.a[0] = (f2d(H[0]) + f2d(Lo[0])) + bx;
+        r.a[1] = (f2d(H[1]) + f2d(Lo[1])) + by;
+        r.a[2] = (f2d(H[2]) + f2d(Lo[2])) + bz;
     } else {
-        const double4_32a I = make_double4_32a(L.x[0], L.x[1], L.x[2], L.m);
-        const double4_32a IA = make_double4_32a(ai[0], ai[1], ai[2], 0.0);
+        const double4_32a I = make_double4_32a(L.x[0], L.x[1], L.x[2], L.md);
+        const double4_32a IA = make_double4_32a(a.a[0], a.a[1], a.a[2], 0.0);
+        r.a[0] = r.a[1] = r.a[2] = 0.0;
         unsigned M = U;
         while (M) {
             const int j = __ffs(M) - 1;
             M &= M - 1;
-            double4_32a J = make_double4_32a(wshd(L.x[0], j), wshd(L.x[1], j), wshd(L.x[2], j), wshd(L.m, j));
-            const double4_32a JA = make_double4_32a(wshd(ai[0], j), wshd(ai[1], j), wshd(ai[2], j), 0.0);
+            double4_32a J = make_double4_32a(wshd(L.x[0], j), wshd(L.x[1], j), wshd(L.x[2], j), wshd(L.md, j));
+            const double4_32a JA = make_double4_32a(wshd(a.a[0], j), wshd(a.a[1], j), wshd(a.a[2], j), 0.0);
             if (!((mysrc >> j) & 1u)) J.w = 0.0;
-            grad_fp64_j<true>(J, JA, I, IA, p.eps2, j, lane, res[0], res[1], res[2]);
+            grad_fp64_j<true>(J, JA, I, IA, L.eps2, j, lane, r.a[0], r.a[1], r.a[2]);
         }
     }
-    for (int q = 0; q < 3; ++q) g[q] = 2.0 * p.G * res[q];
+    return r;
 }
 
 // symmetrised time-step of the lane's particle over the set P (lane in P)
 template <bool MIXED, int SYM>
-__device__ __noinline__ double w_tstep(const SubParams &p, const WLane &L, unsigned P, bool &coincident)
+__device__ __forceinline__ double w_tstep(const SubParams &p, const WLane &L, unsigned P, bool &coincident)
 {
     const int lane = threadIdx.x & 31;
     const int ipos[1] = {lane};
@@ -884,8 +962,8 @@ __device__ __noinline__ double w_tstep(const SubParams &p, const WLane &L, unsig
     // exact fly-by derivative: the lanes' accelerations due to the set
     double la[3] = {0.0, 0.0, 0.0};
     if (SYM & 4) {
-        float wm;
-        w_acc<MIXED>(p, L, P, ((P >> lane) & 1u) ? P : 0u, false, la, wm);
+        const WSum r = w_accel<MIXED, false>(p, L, P, ((P >> lane) & 1u) ? P : 0u);
+        for (int c = 0; c < 3; ++c) la[c] = r.a[c];
     }
     if (MIXED) {
         TstepMixedI<1> I;
@@ -894,11 +972,11 @@ __device__ __noinline__ double w_tstep(const SubParams &p, const WLane &L, unsig
         I.xl[0] = L.rl[0];
         I.yl[0] = L.rl[1];
         I.zl[0] = L.rl[2];
-        I.vx[0] = (float)L.v[0]; I.vy[0] = (float)L.v[1]; I.vz[0] = (float)L.v[2];
-        I.gm[0] = (p.G == 1.0) ? L.mf : (float)(p.G * L.m);
-        I.ax[0] = (float)la[0]; I.ay[0] = (float)la[1]; I.az[0] = (float)la[2];
+        I.vx[0] = d2f(L.v[0]); I.vy[0] = d2f(L.v[1]); I.vz[0] = d2f(L.v[2]);
+        I.gm[0] = (p.G == 1.0) ? L.mf : d2f(p.G * L.m);
+        I.ax[0] = d2f(la[0]); I.ay[0] = d2f(la[1]); I.az[0] = d2f(la[2]);
         const float mf = L.mf;
-        const float eta = (float)p.eta, eta15 = 1.5f * eta;
+        const float eta = p.etaf, eta15 = 1.5f * eta;
         float best[1] = {INFINITY}, minr2[1] = {INFINITY};
         unsigned M = P;
         while (M) {
@@ -912,7 +990,7 @@ __device__ __noinline__ double w_tstep(const SubParams &p, const WLane &L, unsig
             tstep_mixed_j<1, SYM, true>(J0, J1, JV, JA, I, eta, eta15, j, ipos, best, minr2);
         }
         coincident = (minr2[0] == 0.f);
-        return p.eta * (double)best[0];
+        return p.eta * f2d(best[0]);
     } else {
         const double4_32a I = make_double4_32a(L.x[0], L.x[1], L.x[2], L.m);
         const double4_32a IV = make_double4_32a(L.v[0], L.v[1], L.v[2], p.G * L.m);
@@ -936,6 +1014,7 @@ __device__ __noinline__ double w_tstep(const SubParams &p, const WLane &L, unsig
 __device__ __forceinline__ void w_kick(WLane &L, bool on, const double (&a)[3], double dt)
 {
     if (on)
+#pragma unroll
         for (int c = 0; c < 3; ++c) L.v[c] = __dadd_rn(L.v[c], __dmul_rn(dt, a[c]));
 }
 
@@ -956,7 +1035,8 @@ __device__ __forceinline__ void w_drift(WLane &L, bool on, double dt)
 // between the two fsi(S) of one hhs_fsi call, and the frames in between only touch the lanes
 // of F, which are not in S (the same a^SS, bit for bit, as a new pass)
 template <bool MIXED>
-__device__ void w_fsi(const SubParams &p, WLane &L, unsigned S, const StepK &kc, Counts &cnt, int cache = 0)
+__device__ __forceinline__ void w_fsi(const SubParams &p, WLane &L, unsigned S, const StepK &kc, Counts &cnt,
+                                      int cache = 0)
 {
     const double dt = kc.h;
     if (!S) return;
@@ -964,28 +1044,34 @@ __device__ void w_fsi(const SubParams &p, WLane &L, unsigned S, const StepK &kc,
     const bool in = (S >> lane) & 1u;
     const unsigned src = in ? S : 0u;
     const unsigned long long ns = (unsigned long long)__popc(S);
-    if (ns < 2) cache = 0;
-    double a[3], at[3], g[3];
-    float wm;
-    if (cache == 2) {
-        for (int q = 0; q < 3; ++q) a[q] = L.ac[q];
-    } else {
-        w_acc<MIXED>(p, L, S, src, false, a, wm);
+    if (lane == 0) cnt.fsi += 1;
+    if (ns < 2) {
+        // a particle alone: its accelerations are zero and the kicks change nothing
+        w_drift<MIXED>(L, in, 0.5 * dt);
+        w_drift<MIXED>(L, in, 0.5 * dt);
+        return;
     }
-    w_kick(L, in, a, kc.k6);
+    WSum a;
+    if (cache == 2) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) a.a[q] = L.ac[q];
+    } else {
+        a = w_accel<MIXED, false>(p, L, S, src);
+    }
+    w_kick(L, in, a.a, kc.k6);
     w_drift<MIXED>(L, in, 0.5 * dt);
-    w_acc<MIXED>(p, L, S, src, true, a, wm);
-    w_grad<MIXED>(p, L, S, src, a, MIXED ? SLOT_FRACTION * wm : INFINITY, g);
-    const double c = kc.k48;
-    for (int q = 0; q < 3; ++q) at[q] = a[q] + c * g[q];
-    w_kick(L, in, at, kc.k23);
+    a = w_accel<MIXED, true>(p, L, S, src);
+    const WSum g = w_grad<MIXED>(w_src<MIXED>(p, L), S, src, a);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) a.a[q] = grad_kick(p, a.a[q], kc.k48, kc.k24, g.a[q]);
+    w_kick(L, in, a.a, kc.k23);
     w_drift<MIXED>(L, in, 0.5 * dt);
-    w_acc<MIXED>(p, L, S, src, false, a, wm);
+    a = w_accel<MIXED, false>(p, L, S, src);
     if (cache == 1 && in)
-        for (int q = 0; q < 3; ++q) L.ac[q] = a[q];
-    w_kick(L, in, a, kc.k6);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) L.ac[q] = a.a[q];
+    w_kick(L, in, a.a, kc.k6);
     if (lane == 0) {
-        cnt.fsi += 1;
         cnt.acc += (cache == 2 ? 2 : 3) * ns * (ns - 1);
         cnt.grad += ns * (ns - 1);
         if (cache == 2) cnt.reused += ns * (ns - 1);
@@ -993,8 +1079,8 @@ __device__ void w_fsi(const SubParams &p, WLane &L, unsigned S, const StepK &kc,
 }
 
 template <bool MIXED>
-__device__ void w_kick_sf(const SubParams &p, WLane &L, unsigned S, unsigned F, double cdt, bool gradient,
-                          double c48, Counts &cnt)
+__device__ __forceinline__ void w_kick_sf(const SubParams &p, WLane &L, unsigned S, unsigned F, double cdt,
+                                          bool gradient, const StepK &kc, Counts &cnt)
 {
     if (!S || !F) return;
     const int lane = threadIdx.x & 31;
@@ -1002,15 +1088,16 @@ __device__ void w_kick_sf(const SubParams &p, WLane &L, unsigned S, unsigned F, 
     const unsigned src = inS ? F : (inF ? S : 0u);
     const unsigned U = S | F;
     const unsigned long long pairs = 2ull * __popc(S) * __popc(F);
-    double a[3];
-    float wm;
-    w_acc<MIXED>(p, L, U, src, gradient, a, wm);
+    WSum a;
     if (gradient) {
-        double g[3];
-        w_grad<MIXED>(p, L, U, src, a, MIXED ? SLOT_FRACTION * wm : INFINITY, g);
-        for (int q = 0; q < 3; ++q) a[q] = a[q] + c48 * g[q];
+        a = w_accel<MIXED, true>(p, L, U, src);
+        const WSum g = w_grad<MIXED>(w_src<MIXED>(p, L), U, src, a);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) a.a[q] = grad_kick(p, a.a[q], kc.k48, kc.k24, g.a[q]);
+    } else {
+        a = w_accel<MIXED, false>(p, L, U, src);
     }
-    w_kick(L, inS || inF, a, cdt);
+    w_kick(L, inS || inF, a.a, cdt);
     if (lane == 0) {
         cnt.acc += pairs;
         if (gradient) cnt.grad += pairs;
@@ -1096,7 +1183,7 @@ __device__ __noinline__ int warp_hhs(const SubParams &p, const int32_t *Sg, int 
                 atomicAdd(&p.levels[SUBTREE_STAT_LEVELS + Lv], np);
             }
             const StepK &K0 = p.K[depth - p.kdepth0];
-            w_kick_sf<MIXED>(p, L, Sn, Fn, K0.k6, false, K0.k48, cnt);
+            w_kick_sf<MIXED>(p, L, Sn, Fn, K0.k6, false, K0, cnt);
             w_fsi<MIXED>(p, L, Sn, p.K[depth - p.kdepth0 + 1], cnt, 1);
             if (lane == 0) {
                 wf_S[top] = Sn;
@@ -1118,7 +1205,7 @@ __device__ __noinline__ int warp_hhs(const SubParams &p, const int32_t *Sg, int 
             }
         } else if (pc == 1) {
             const StepK &K0 = p.K[depth - p.kdepth0];
-            w_kick_sf<MIXED>(p, L, S, F, K0.k23, true, K0.k48, cnt);
+            w_kick_sf<MIXED>(p, L, S, F, K0.k23, true, K0, cnt);
             if (lane == 0) wf_pc[top] = 2;
             if (F) {
                 if (lane == 0) {
@@ -1133,7 +1220,7 @@ __device__ __noinline__ int warp_hhs(const SubParams &p, const int32_t *Sg, int 
         } else {
             const StepK &K0 = p.K[depth - p.kdepth0];
             w_fsi<MIXED>(p, L, S, p.K[depth - p.kdepth0 + 1], cnt, 2);
-            w_kick_sf<MIXED>(p, L, S, F, K0.k6, false, K0.k48, cnt);
+            w_kick_sf<MIXED>(p, L, S, F, K0.k6, false, K0, cnt);
             sp -= 1;
         }
         __syncwarp();
@@ -1206,7 +1293,7 @@ __global__ void __launch_bounds__(SB, MINB) k_hhs_subtree(SubParams p0, SubWork 
     if (tid <= MAXD) {
         const double sc = __longlong_as_double((long long)(1023 - tid) << 52);  // 2^-tid
         const double k6 = tau0 / 6.0, k23 = 2.0 * tau0 / 3.0, k48 = tau0 * tau0 / 48.0;
-        s_K[tid] = StepK{tau0 * sc, k6 * sc, k23 * sc, k48 * (sc * sc)};
+        s_K[tid] = StepK{tau0 * sc, k6 * sc, k23 * sc, k48 * (sc * sc), 2.0 * (k48 * (sc * sc))};
     }
     p.K = s_K;
     p.kdepth0 = depth0;
@@ -1391,6 +1478,9 @@ cudaError_t launch_subtree(cudaStream_t s, bool mixed, int sym, const SubtreeArg
     p.G = a.G;
     p.eta = a.eta;
     p.eps2 = a.eps2;
+    p.eps2f = (float)a.eps2;
+    p.etaf = (float)a.eta;
+    p.unit_G = a.G == 1.0 ? 1 : 0;
     p.max_depth = a.max_depth;
     p.err = a.err;
     p.counters = a.counters;
