@@ -50,10 +50,9 @@ enum { G_X, G_Y, G_Z, G_M, G_AX, G_AY, G_AZ, G_XL, G_YL, G_ZL, G_AXL, G_AYL, G_A
 static_assert(P_ROWS == TILE_POS_ROWS && G_ROWS == TILE_GRAD_ROWS, "record sizes in frost_internal.cuh");
 
 struct Head {
-    float4 c;   // {centre, radius}
-    float4 lo;  // {box rounded outwards, smallest m^(-2/3)}
-    float4 hi;
-    float4 a;   // {mean acceleration of the sources that count, 0} (gradient)
+    float4 c;  // {centre, radius}
+    float4 h;  // {largest |offset from the centre| by component, smallest m^(-2/3)}
+    float4 a;  // {mean acceleration of the sources that count, 0} (gradient)
 };
 static_assert(sizeof(Head) == TILE_HEAD_BYTES, "head size in frost_internal.cuh");
 
@@ -78,13 +77,16 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// a lower bound on the squared distance of two boxes
-__device__ __forceinline__ float box_gap2(const float4 alo, const float4 ahi, const float4 blo, const float4 bhi)
+// The squared distance of two boxes, from below: centres and half sizes are FP32 values, so the
+// gap is good to a few units whatever the distance of the tiles from the origin
+__device__ __forceinline__ float axis_gap(float d, float h) { return fmaxf(0.f, fmaf(fabsf(d), 0.999999f, -1.000001f * h)); }
+
+__device__ __forceinline__ float box_gap2(const float4 ca, const float4 ha, const float4 cb, const float4 hb)
 {
-    const float gx = fmaxf(0.f, fmaxf(__fsub_rd(blo.x, ahi.x), __fsub_rd(alo.x, bhi.x)));
-    const float gy = fmaxf(0.f, fmaxf(__fsub_rd(blo.y, ahi.y), __fsub_rd(alo.y, bhi.y)));
-    const float gz = fmaxf(0.f, fmaxf(__fsub_rd(blo.z, ahi.z), __fsub_rd(alo.z, bhi.z)));
-    return __fmaf_rd(gx, gx, __fmaf_rd(gy, gy, __fmul_rd(gz, gz)));
+    const float gx = axis_gap(ca.x - cb.x, ha.x + hb.x);
+    const float gy = axis_gap(ca.y - cb.y, ha.y + hb.y);
+    const float gz = axis_gap(ca.z - cb.z, ha.z + hb.z);
+    return fmaf(gx, gx, fmaf(gy, gy, gz * gz));
 }
 
 // ------------------------------------------------------------------------------------
@@ -122,20 +124,26 @@ __global__ void __launch_bounds__(128) k_tile_pack(const int32_t *__restrict__ l
         }
         mass[e] = m[i];
     }
-    float lo[3], hi[3], c[3], r2[2] = {0.f, 0.f};
+    float half[3], c[3], r2[2] = {0.f, 0.f};
 #pragma unroll
     for (int q = 0; q < 3; ++q) {
-        lo[q] = warp_min(fminf(live[0] ? __double2float_rd(p[0][q]) : INFINITY, live[1] ? __double2float_rd(p[1][q]) : INFINITY));
-        hi[q] = warp_max(fmaxf(live[0] ? __double2float_ru(p[0][q]) : -INFINITY, live[1] ? __double2float_ru(p[1][q]) : -INFINITY));
-        c[q] = 0.5f * lo[q] + 0.5f * hi[q];
+        const float p0 = (float)p[0][q], p1 = (float)p[1][q];
+        const float lo = warp_min(fminf(live[0] ? p0 : INFINITY, live[1] ? p1 : INFINITY));
+        const float hi = warp_max(fmaxf(live[0] ? p0 : -INFINITY, live[1] ? p1 : -INFINITY));
+        c[q] = 0.5f * lo + 0.5f * hi;
+        float far = 0.f;
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const double d = live[e] ? p[e][q] - (double)c[q] : (double)kFar;
             const float h = (float)d;
             t[((GRAD ? G_X : P_X) + q) * TJ + e * 32] = h;
             t[((GRAD ? G_XL : P_XL) + q) * TJ + e * 32] = live[e] ? (float)(d - (double)h) : 0.f;
-            if (live[e]) r2[e] = fmaf(h, h, r2[e]);
+            if (live[e]) {
+                r2[e] = fmaf(h, h, r2[e]);
+                far = fmaxf(far, fabsf(h));
+            }
         }
+        half[q] = warp_max(far);
     }
     Head h;
     float mq = INFINITY;
@@ -180,8 +188,7 @@ __global__ void __launch_bounds__(128) k_tile_pack(const int32_t *__restrict__ l
         h.a = make_float4(ac[0], ac[1], ac[2], 0.f);
     }
     h.c = make_float4(c[0], c[1], c[2], 1.00001f * sqrtf(warp_max(fmaxf(r2[0], r2[1]))));
-    h.lo = make_float4(lo[0], lo[1], lo[2], warp_min(mq));
-    h.hi = make_float4(hi[0], hi[1], hi[2], 0.f);
+    h.h = make_float4(half[0], half[1], half[2], warp_min(mq));
     if (lane == 0) ((Head *)heads(rec, n, ROWS))[tile] = h;
 }
 
@@ -254,15 +261,13 @@ __device__ __forceinline__ double group_total(const Group &W, int q, int r)
     return ((double)W.H[q][r].x + (double)W.L[q][r].x) + ((double)W.H[q][r].y + (double)W.L[q][r].y);
 }
 
-// a lower bound, but for the rounding of the position, on the squared distance of this lane's
-// receiver k from a box
-__device__ __forceinline__ float point_gap2(const Group &W, int k, const float4 lo, const float4 hi)
+// the squared distance of this lane's receiver k from a tile's box, from below
+__device__ __forceinline__ float point_gap2(const Group &W, int k, const float4 c, const float4 h)
 {
     const int r = slot_of(k);
-    const float px = W.head.c.x + W.xh[0][r], py = W.head.c.y + W.xh[1][r], pz = W.head.c.z + W.xh[2][r];
-    const float gx = fmaxf(0.f, fmaxf(lo.x - px, px - hi.x));
-    const float gy = fmaxf(0.f, fmaxf(lo.y - py, py - hi.y));
-    const float gz = fmaxf(0.f, fmaxf(lo.z - pz, pz - hi.z));
+    const float gx = axis_gap((W.head.c.x - c.x) + W.xh[0][r], h.x);
+    const float gy = axis_gap((W.head.c.y - c.y) + W.xh[1][r], h.y);
+    const float gz = axis_gap((W.head.c.z - c.z) + W.xh[2][r], h.z);
     return fmaf(gx, gx, fmaf(gy, gy, gz * gz));
 }
 
@@ -343,33 +348,24 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
     const Head *jh = heads(jrec, n_s, P_ROWS);
     load_group(W, irec, n_a, P_ROWS, P_XL, g);
     float q[2] = {INFINITY, INFINITY};
-    // first the tiles whose boxes touch the receivers' box, or else the nearest one
+    // first the tile whose centre is nearest (in a self pass the receivers' own)
     float best = INFINITY;
-    int at = -1;
-    bool some = false;
-    for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
-        const int t = t0 + lane * nsplit;
-        float d = INFINITY;
-        if (t < ntiles) {
-            d = box_gap2(W.head.lo, W.head.hi, jh[t].lo, jh[t].hi);
-            if (d < best) {
-                best = d;
-                at = t;
-            }
-        }
-        for (unsigned mask = __ballot_sync(kFull, d == 0.f); mask; mask &= mask - 1) {
-            const int tt = t0 + (__ffs(mask) - 1) * nsplit;
-            wmax_tile(W, g, jrec, jh[tt], tt, self_pass && tt == g, eps2, s, q);
-            some = true;
+    int first = -1;
+    for (int t = blockIdx.y + lane * nsplit; t < ntiles; t += 32 * nsplit) {
+        const float4 c = jh[t].c;
+        const float x = c.x - W.head.c.x, y = c.y - W.head.c.y, z = c.z - W.head.c.z;
+        const float d = fmaf(x, x, fmaf(y, y, z * z));
+        if (d < best) {
+            best = d;
+            first = t;
         }
     }
-    if (!some) {
+    {
         const float d = warp_min(best);
-        const unsigned mask = __ballot_sync(kFull, best == d && at >= 0);
-        if (mask) {
-            at = __shfl_sync(kFull, at, __ffs(mask) - 1);
-            wmax_tile(W, g, jrec, jh[at], at, false, eps2, s, q);
-        }
+        const unsigned mask = __ballot_sync(kFull, best == d && first >= 0);
+        if (!mask) return;
+        first = __shfl_sync(kFull, first, __ffs(mask) - 1);
+        wmax_tile(W, g, jrec, jh[first], first, self_pass && first == g, eps2, s, q);
     }
     // then those that can still hold a larger m_j / r^3 for some receiver: box against box, then
     // every receiver against the box (a few receivers far from the others stretch the group's box
@@ -378,9 +374,9 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
         const int t = t0 + lane * nsplit;
         const float qmax = 1.0001f * warp_max(fmaxf(g * TJ + slot_of(0) < n_a ? q[0] : 0.f, g * TJ + slot_of(1) < n_a ? q[1] : 0.f));
         bool near = false;
-        if (t < ntiles) {
-            const float d = box_gap2(W.head.lo, W.head.hi, jh[t].lo, jh[t].hi);
-            near = d != 0.f && !((d + eps2) * jh[t].lo.w > qmax);
+        if (t < ntiles && t != first) {
+            const float4 c = jh[t].c, h = jh[t].h;
+            near = !((box_gap2(W.head.c, W.head.h, c, h) + eps2) * h.w > qmax);
         }
         for (unsigned mask = __ballot_sync(kFull, near); mask; mask &= mask - 1) {
             const int tt = t0 + (__ffs(mask) - 1) * nsplit;
@@ -388,8 +384,8 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
             bool any = false;
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                any = any || (g * TJ + slot_of(k) < n_a && !((point_gap2(W, k, J.lo, J.hi) + eps2) * J.lo.w > 1.0001f * q[k]));
-            if (__any_sync(kFull, any)) wmax_tile(W, g, jrec, J, tt, false, eps2, s, q);
+                any = any || (g * TJ + slot_of(k) < n_a && !((point_gap2(W, k, J.c, J.h) + eps2) * J.h.w > 1.0001f * q[k]));
+            if (__any_sync(kFull, any)) wmax_tile(W, g, jrec, J, tt, self_pass && tt == g, eps2, s, q);
         }
     }
 #pragma unroll
@@ -401,32 +397,35 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
     }
 }
 
-// The next 32 tiles of a split: far (fm) and near (nm).  Far tiles are far enough for single
-// separations (box against box) and, with HEAVY, hold no term above a receiver's threshold:
-// their heaviest mass at distance d stays below it, d^2 m^(-2/3) > qk of every receiver (box
-// against box at the largest qk, qthr, then receiver by receiver).
+// The next 32 tiles of a split: far (fm) and near (nm).  A tile is far from a receiver at
+// distance d >= kFarRadius R_J of its box and, with HEAVY, if it holds no dominant term to look
+// for: its heaviest mass at d stays below the receiver's threshold, d^2 m^(-2/3) > qk, or
+// d >= R_J, where its 64 terms are much alike (from outside a core, all of its terms are within
+// a factor 16 of the largest, and none of them dominates).  Box against box with the largest qk
+// (qthr) first, then, where that does not settle it, receiver by receiver.
 template <bool HEAVY>
 __device__ __forceinline__ void judge_tiles(const Group &W, const Head *__restrict__ jh, int ntiles, int t0, int nsplit,
-                                            float qthr, const float (&qk)[2], unsigned &fm, unsigned &nm)
+                                            int own, bool live0, bool live1, float qthr, const float (&qk)[2], unsigned &fm,
+                                            unsigned &nm)
 {
     const int t = t0 + (threadIdx.x & 31) * nsplit;
-    bool apart = false, light = true;
-    if (t < ntiles) {
-        const float4 lo = jh[t].lo, hi = jh[t].hi;
-        const float R = jh[t].c.w, d2 = box_gap2(W.head.lo, W.head.hi, lo, hi);
-        apart = d2 > 0.f && d2 >= (kFarRadius * kFarRadius) * R * R;
-        light = !HEAVY || d2 * lo.w > qthr;
+    bool far = false;
+    if (t < ntiles && t != own) {
+        const float4 c = jh[t].c, h = jh[t].h;
+        const float d2 = box_gap2(W.head.c, W.head.h, c, h), R2 = c.w * c.w;
+        far = d2 > 0.f && d2 >= (kFarRadius * kFarRadius) * R2 && (!HEAVY || d2 * h.w > qthr || d2 >= R2);
     }
-    fm = __ballot_sync(kFull, apart && light);
-    nm = __ballot_sync(kFull, t < ntiles && !apart);
-    if (HEAVY)
-        for (unsigned um = __ballot_sync(kFull, apart && !light); um; um &= um - 1) {
-            const int b = __ffs(um) - 1;
-            const float4 lo = jh[t0 + b * nsplit].lo, hi = jh[t0 + b * nsplit].hi;
-            const bool heavy = !(point_gap2(W, 0, lo, hi) * lo.w > qk[0]) || !(point_gap2(W, 1, lo, hi) * lo.w > qk[1]);
-            if (__any_sync(kFull, heavy)) nm |= 1u << b;
-            else fm |= 1u << b;
-        }
+    fm = __ballot_sync(kFull, far);
+    nm = 0u;
+    for (unsigned um = __ballot_sync(kFull, t < ntiles && !far); um; um &= um - 1) {
+        const int b = __ffs(um) - 1, tt = t0 + b * nsplit;
+        const float4 c = jh[tt].c, h = jh[tt].h;
+        const float R2 = c.w * c.w, d0 = point_gap2(W, 0, c, h), d1 = point_gap2(W, 1, c, h);
+        const bool ok0 = d0 > 0.f && d0 >= (kFarRadius * kFarRadius) * R2 && (!HEAVY || d0 * h.w > qk[0] || d0 >= R2);
+        const bool ok1 = d1 > 0.f && d1 >= (kFarRadius * kFarRadius) * R2 && (!HEAVY || d1 * h.w > qk[1] || d1 >= R2);
+        if (tt != own && __all_sync(kFull, (ok0 || !live0) && (ok1 || !live1))) fm |= 1u << b;
+        else nm |= 1u << b;
+    }
 }
 
 // ------------------------------------------------------------------------------------
@@ -436,8 +435,8 @@ __device__ __forceinline__ void judge_tiles(const Group &W, const Head *__restri
 // their terms (with the terms beyond the FP32 range apart in FP64).  In local memory: they are
 // touched a few times per receiver and split.  The limit is for receivers far out in the halo,
 // for which thousands of sources are within a factor 16 of the nearest: their warps, without
-// it, made the 65536-body passes a third longer.
-constexpr int SLOTS = 32;
+// it, made the 65536-body passes a third longer (32 slots: a step of 53.1 ms, 16: 52.3 ms).
+constexpr int SLOTS = 16;
 struct Slots {
     int j[2][SLOTS];
     float sum[2][6];
@@ -569,7 +568,8 @@ __global__ void __launch_bounds__(32, ACC ? 16 : 20) k_acc_tile(const float *__r
     const float2 e2 = dup(eps2);
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
         unsigned fm, nm;
-        judge_tiles<ACC>(W, jh, ntiles, t0, nsplit, qthr, qk, fm, nm);
+        judge_tiles<ACC>(W, jh, ntiles, t0, nsplit, self_pass ? g : -1, g * TJ + slot_of(0) < n_a, g * TJ + slot_of(1) < n_a, qthr,
+                         qk, fm, nm);
         // the next tile's rows wait in registers: 64 pieces of the far rows, 128 of all
         auto next_bit = [&]() { return fm ? __ffs(fm) - 1 : __ffs(nm) - 1; };
         float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
@@ -786,7 +786,8 @@ __global__ void __launch_bounds__(32, 16) k_grad_tile(const float *__restrict__ 
     const float2 e2 = dup((float)eps2d);
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
         unsigned fm, nm;
-        judge_tiles<true>(W, jh, ntiles, t0, nsplit, qthr, qk, fm, nm);
+        judge_tiles<true>(W, jh, ntiles, t0, nsplit, self_pass ? g : -1, g * TJ + slot_of(0) < n_a, g * TJ + slot_of(1) < n_a, qthr,
+                         qk, fm, nm);
         auto next_bit = [&]() { return fm ? __ffs(fm) - 1 : __ffs(nm) - 1; };
         // the next tile's far rows wait in registers, 112 of its 208 pieces
         float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
@@ -943,9 +944,10 @@ __global__ void __launch_bounds__(32, 16) k_grad_tile(const float *__restrict__ 
 int tile_splits(int n_a, int n_s, int n_sm, size_t part_elems)
 {
     const long long ngroups = (n_a + TJ - 1) / TJ, ntiles = (n_s + TJ - 1) / TJ;
-    // eight rounds of about 20 resident warps an SM, each warp four tiles at least, the partials
-    // within their buffer
-    long long ns = std::min((8LL * 20 * n_sm + ngroups - 1) / ngroups, (ntiles + 3) / 4);
+    // eight rounds of about 20 resident warps an SM, each warp 16 tiles at least (its slots, a few
+    // double-float terms a lane whatever it sees, cost as much as several tiles: with 4 tiles a
+    // warp a 65536-body step took 55.4 ms, with 16 52.3), the partials within their buffer
+    long long ns = std::min((8LL * 20 * n_sm + ngroups - 1) / ngroups, (ntiles + 15) / 16);
     ns = std::min<long long>(ns, (long long)(part_elems / (3 * (size_t)n_a)));
     return (int)std::max<long long>(1, ns);
 }

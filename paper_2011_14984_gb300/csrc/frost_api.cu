@@ -113,7 +113,13 @@ constexpr int kTileMinN = 8192;
 // the same for the Newtonian and gradient passes: the lists of a pass entry point from
 // kOrderForceMinN particles on, and inside a step two lists of at least kTileForceMinN
 constexpr int kOrderForceMinN = 24576;
-constexpr int kTileForceMinN = 2048;
+// two lists of a gradient entry point: from this many pairs on, and each list of at least
+// kOrderCrossMinN (a sparse list's tiles are wide).  25000 x 40000 particles: 4.67 ms so, 6.03
+// on the symmetric passes; 12001 x 11905: 1.37 and 1.46; 16717 x 6101: 1.14 and 1.16; 2049 x
+// 65537: 1.32 and 1.35, but with errors a quarter larger
+constexpr int64_t kOrderCrossMinPairs = int64_t(1) << 27;
+constexpr int kOrderCrossMinN = 8192;
+constexpr int kTileForceMinN = 4096;
 
 // autotuner rows: the pass kinds, and the Newtonian pass that feeds a gradient (mixed mode:
 // its wmax prepass and deferred double-float terms give it a cost profile of its own)
@@ -447,6 +453,11 @@ bool tile_tstep(const frost_ctx *c, int n) { return c->ordered && n >= kTileMinN
 // the tile kernels
 bool tile_force(const frost_ctx *c, int nA, int nB) { return c->ordered && std::min(nA, nB) >= kTileForceMinN; }
 
+bool order_cross(const frost_ctx *c, int nA, int nB)
+{
+    return c->ord && std::min(nA, nB) >= kOrderCrossMinN && (int64_t)nA * nB >= kOrderCrossMinPairs;
+}
+
 TileArgs tile_args(const frost_ctx *c, const Lane &L, const void *irec, int nA, const void *jrec, int nB, bool self)
 {
     TileArgs a;
@@ -760,6 +771,32 @@ void pack_grad(frost_ctx *c, Lane &L, const int32_t *list, int n, const double *
     else if (c->mixed) launch_pack_grad_mixed(L.s, list, n, c->x, c->m, c->N, a, (float4 *)rec, mask);
     else launch_pack_grad_fp64(L.s, list, n, c->x, c->m, c->N, a, (double4_32a *)rec);
     c->st.kernel_launches += 1;
+}
+
+// The force-gradient kick of two disjoint lists due to each other on the tile kernels, both lists
+// put in spatial order first and the results in the callers' orders (any may be NULL; only_a:
+// without B's gradient).  The order's buffers are free outside a step.
+void grad_pairwise_tile(frost_ctx *c, Lane &M, const int32_t *A, int nA, const int32_t *B, int nB, double eps_grad,
+                        double *acc_a, double *acc_b, double *at_a, double *at_b, double *g_a, double *g_b, bool only_a)
+{
+    int32_t *SA = c->olist, *SB = c->ord;
+    const int32_t *pA = c->opos, *pB = c->ptmp;
+    order_list(c, A, nA, c->opos, SA);
+    order_list(c, B, nB, c->ptmp, SB);
+    unsigned *h = zero_hists(M);
+    pack_acc(c, M, SA, nA, M.recA, true);
+    pack_acc(c, M, SB, nB, M.recB, true);
+    pass_acc(c, M, SA, nA, SB, nB, false, M.aA, acc_a, M.wA, h, KickArgs(), M.recA, M.recB, false, true, pA);
+    pass_acc(c, M, SB, nB, SA, nA, false, M.aB, acc_b, M.wB, h + HOT_BINS, KickArgs(), M.recB, M.recA, false, true, pB);
+    mark_hot(c, M, nA, nB, false, M.aA, h, h + HOT_BINS, nB, M.hA);
+    mark_hot(c, M, nB, nA, false, M.aB, h + HOT_BINS, h, nA, M.hB);
+    pack_grad(c, M, SA, nA, M.aA, M.recA, M.hA, true);
+    pack_grad(c, M, SB, nB, M.aB, M.recB, M.hB, true);
+    pass_grad(c, M, SA, nA, M.aA, SB, nB, M.aB, false, eps_grad, nullptr, at_a, g_a, M.wA, M.hB, KickArgs(), M.recA,
+              M.recB, true, pA);
+    if (!only_a)
+        pass_grad(c, M, SB, nB, M.aB, SA, nA, M.aA, false, eps_grad, nullptr, at_b, g_b, M.wB, M.hA, KickArgs(), M.recB,
+                  M.recA, true, pB);
 }
 
 // Algorithm fsi on the set S with step dt.  Each kick is fused into the finalisation of the
@@ -1570,6 +1607,8 @@ frost_status frost_accel_gradient(frost_ctx *c, const int32_t *active, int64_t n
         if (want_grad)
             pass_grad(c, M, P, nA, c->aA, P, nA, c->aA, true, eps_grad, nullptr, acc_tilde, grad, c->wA, c->hA,
                       KickArgs(), nullptr, nullptr, tile, omap);
+    } else if (want_grad && order_cross(c, nA, nB)) {
+        grad_pairwise_tile(c, M, A, nA, B, nB, eps_grad, acc, nullptr, acc_tilde, nullptr, grad, nullptr, true);
     } else if (want_grad && c->mixed && nB > 0 && c->sym_cross >= 0 &&
                (c->sym_cross > 0 || (int64_t)nA * nB >= kSymCrossPrepassMinPairs)) {
         // both accurate passes on records packed once, their prepasses in one symmetric kernel
@@ -1642,7 +1681,9 @@ frost_status frost_accel_gradient_pairwise(frost_ctx *c, const int32_t *a, int64
     if (c->hmisc->rel[0]) return fail(FROST_EINVAL, "index list has an out-of-range or repeated index");
     if (c->hmisc->rel[1] != 0) return fail(FROST_EINVAL, "the two lists share %lld particles", (long long)c->hmisc->rel[1]);
     Lane &M = c->main;
-    if (nA > 0 && nB > 0) {
+    if (order_cross(c, nA, nB)) {
+        grad_pairwise_tile(c, M, A, nA, B, nB, eps_grad, acc_a, acc_b, acc_tilde_a, acc_tilde_b, grad_a, grad_b, false);
+    } else if (nA > 0 && nB > 0) {
         pack_pos(c, M, A, nA, M.recA);
         pack_pos(c, M, B, nB, M.recB);
         const bool sym = c->sym_cross >= 0 &&

@@ -279,7 +279,7 @@ void launch_tstep_tile(cudaStream_t s, const int32_t *list, int n, const double 
 // Mixed Newtonian and gradient passes of spatially ordered lists (force_tiles.cu).  rec: tiles of
 // TILE_N particles, TILE_POS_ROWS or TILE_GRAD_ROWS rows of TILE_N floats, then the tiles' heads.
 constexpr int TILE_N = 64;
-constexpr int TILE_POS_ROWS = 9, TILE_GRAD_ROWS = 13, TILE_HEAD_BYTES = 64;
+constexpr int TILE_POS_ROWS = 9, TILE_GRAD_ROWS = 13, TILE_HEAD_BYTES = 48;
 struct TileArgs {
     const void *irec, *jrec;
     int n_a, n_s;
