@@ -103,11 +103,12 @@ typedef struct {
                                result bits: the pair criteria are symmetric and a minimum does
                                not depend on the order).  1: all always; -1: never.  (Mixed mode,
                                contexts of at least 16384 particles: frost_step orders the
-                               particles in space before every top-level step, and the time-step
-                               passes of large ordered lists, and of lists of at least 16384
-                               particles given to frost_timesteps, look at far groups of
-                               particles through bounds instead, again with the same bits; not
-                               with the exact fly-by derivative.) */
+                               particles in space before every top-level step, and the passes of
+                               large ordered lists, and of large lists given to the entry points,
+                               look at groups of particles through their boxes instead, in every
+                               mode of this option.  Time-steps keep their bits; forces keep the
+                               accuracy stated at frost_accel_gradient.  The exact fly-by
+                               derivative's time-steps stay as they are.) */
 } frost_opts;
 
 typedef enum {
@@ -181,8 +182,8 @@ frost_status frost_get_state(frost_ctx *ctx, double *x, double *v, double *t);
  * With softening eps_P, r^2 -> r^2 + eps_P^2 everywhere in both sums.  Pairs at zero
  * separation give FROST_ECOINCIDENT when unsoftened.  Synchronises.
  * Accuracy: FP64 mode, 1e-12 relative.  Mixed mode: the Newtonian pass runs a prepass for
- * max_j m_j / r^3 and sums the terms above 1/16 of it (up to 8 per particle) in
- * double-float, and so does the gradient pass; the rest are FP32 terms in compensated sums.
+ * max_j m_j / r^3 and sums the terms above 1/16 of it (up to 8 per particle and split of
+ * the sources, 16 in large sets) in double-float, and so does the gradient pass; the rest are FP32 terms in compensated sums.
  * That gives a_i to about 1e-7 and g_i to below 1e-6 at the 99.9th percentile of a set of a
  * few thousand particles or more.  The relative error of one g_i grows as
  * sum_j |term_ij| / |g_i| where the gradient nearly vanishes.

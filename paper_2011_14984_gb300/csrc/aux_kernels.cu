@@ -286,22 +286,21 @@ __global__ void k_check_mass(const double *__restrict__ m, int n, int *__restric
 // relative accuracy per phi_i (positions enter exactly, as three FP32 parts).
 
 // records: p0 = {x_h, y_h, z_h, m_h}, p1 = {x_l, y_l, z_l, m_l}, p2 = {x_ll, y_ll, z_ll, 0}
-__global__ void k_pack_pot_df(const double *__restrict__ x, const double *__restrict__ m, int N,
-                              float4 *__restrict__ rec)
+__global__ void k_pack_pot_df(const int32_t *__restrict__ list, const double *__restrict__ x,
+                              const double *__restrict__ m, int N, float4 *__restrict__ rec)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= N) return;
+    const int i = list ? list[k] : k;
     float xh, xl, xll, yh, yl, yll, zh, zl, zll;
     df::split3(x[i], xh, xl, xll);
     df::split3(x[N + i], yh, yl, yll);
     df::split3(x[2 * N + i], zh, zl, zll);
-    const double pm = m[i];
-    const float hm = (float)pm;
-    rec[i] = make_float4(xh, yh, zh, hm);
-    rec[N + i] = make_float4(xl, yl, zl, (float)(pm - (double)hm));
-    rec[2 * N + i] = make_float4(xll, yll, zll, 0.f);
+    const df::dfloat pm = df::from_double(m[i]);
+    rec[k] = make_float4(xh, yh, zh, pm.h);
+    rec[N + k] = make_float4(xl, yl, zl, pm.l);
+    rec[2 * N + k] = make_float4(xll, yll, zll, 0.f);
 }
-
 
 // phi_i = sum_{j > i} m_j / sqrt(r^2 + eps2) in double-float, j-split partials part[split][i]:
 // each pair once (U = -G sum_i m_i phi_i); the tiles wholly at or below the block's i-range are
@@ -340,29 +339,8 @@ __global__ void __launch_bounds__(BS) k_potential_df(const float4 *__restrict__ 
             const df::dfloat sx = df::sep(J0.x, J1.x, J2.x, I0.x, I1.x, I2.x);
             const df::dfloat sy = df::sep(J0.y, J1.y, J2.y, I0.y, I1.y, I2.y);
             const df::dfloat sz = df::sep(J0.z, J1.z, J2.z, I0.z, I1.z, I2.z);
-            const float xh = sx.h, xl = sx.l, yh = sy.h, yl = sy.l, zh = sz.h, zl = sz.l;
-            // r^2 + eps^2: exact squares of the high parts, first-order terms of the low parts
-            // (products feeding an error-free transformation are rounded on their own, __fmul_rn,
-            // so that the compiler cannot contract them into the following add)
-            const float px = __fmul_rn(xh, xh), py = __fmul_rn(yh, yh), pz = __fmul_rn(zh, zh);
-            const float qx = fmaf(xh + xh, xl, fmaf(xh, xh, -px));
-            const float qy = fmaf(yh + yh, yl, fmaf(yh, yh, -py));
-            const float qz = fmaf(zh + zh, zl, fmaf(zh, zh, -pz));
-            float s, t, S, u, S2, u2;
-            df::two_sum(px, py, s, t);
-            df::two_sum(s, pz, S, u);
-            df::two_sum(S, e2h, S2, u2);
-            const float lo = ((t + u) + (u2 + e2l)) + ((qx + qy) + qz);
-            // 1 / r: MUFU estimate y0 and the residual res = 1 - r^2 y0^2 in double-float; then
-            // 1/r = y0 (1 - res)^(-1/2) = y0 (1 + res/2 + 3 res^2/8 + ...), |res| < 2^-21
-            const float y0 = rsqrtf(S2);
-            const float q = __fmul_rn(y0, y0), qe = fmaf(y0, y0, -q);
-            const float pp = __fmul_rn(S2, q), pe = fmaf(S2, q, -pp);
-            const float res = ((1.f - pp) - pe) - fmaf(S2, qe, lo * q);
-            const float c = y0 * res * fmaf(0.375f, res, 0.5f);
-            // m_j / r = (m_h + m_l)(y0 + c)
-            const float w = __fmul_rn(J0.w, y0);
-            const float we = fmaf(J0.w, y0, -w) + fmaf(J0.w, c, J1.w * y0);
+            float w, we;
+            df::mass_over_r(sx.h, sx.l, sy.h, sy.l, sz.h, sz.l, e2h, e2l, J0.w, J1.w, w, we);
             if (j0 + jj > i) {
                 float e;
                 df::two_sum(H, w, H, e);
@@ -535,9 +513,14 @@ void launch_potential(cudaStream_t s, const double *x, const double *m, int n, d
                       double *part, const SplitShape &shape)
 {
     if (n <= 0) return;
-    k_pack_pot_df<<<cdiv(n, 256), 256, 0, s>>>(x, m, n, rec);
+    k_pack_pot_df<<<cdiv(n, 256), 256, 0, s>>>(nullptr, x, m, n, rec);
     const dim3 grid(shape.nblk_i, shape.nsplit);
     k_potential_df<PAIR_BS, PAIR_TJ><<<grid, PAIR_BS, 0, s>>>(rec, n, shape.j_per_split, eps2, part);
+}
+
+void launch_pack_pot(cudaStream_t s, const int32_t *list, const double *x, const double *m, int n, float4 *rec)
+{
+    if (n > 0) k_pack_pot_df<<<cdiv(n, 256), 256, 0, s>>>(list, x, m, n, rec);
 }
 
 int potential_blocks_per_sm()

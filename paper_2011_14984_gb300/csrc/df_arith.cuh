@@ -147,5 +147,34 @@ __device__ __forceinline__ dfloat sep(float jh, float jl, float jll, float ih, f
     return r;
 }
 
+// m / sqrt(x^2 + y^2 + z^2 + e2) = w + we from the separation's high and low parts (|low| up to a
+// few units of the high part: without their squares, always positive, U would be 2e-15 too large)
+__device__ __forceinline__ void mass_over_r(float xh, float xl, float yh, float yl, float zh, float zl, float e2h,
+                                            float e2l, float mh, float ml, float &w, float &we)
+{
+    // r^2 + eps^2: exact squares of the high parts, (2 high + low) low for the rest
+    // (products feeding an error-free transformation are rounded on their own, __fmul_rn,
+    // so that the compiler cannot contract them into the following add)
+    const float px = __fmul_rn(xh, xh), py = __fmul_rn(yh, yh), pz = __fmul_rn(zh, zh);
+    const float qx = fmaf(fmaf(2.f, xh, xl), xl, fmaf(xh, xh, -px));
+    const float qy = fmaf(fmaf(2.f, yh, yl), yl, fmaf(yh, yh, -py));
+    const float qz = fmaf(fmaf(2.f, zh, zl), zl, fmaf(zh, zh, -pz));
+    float s, t, S, u, S2, u2;
+    two_sum(px, py, s, t);
+    two_sum(s, pz, S, u);
+    two_sum(S, e2h, S2, u2);
+    const float lo = ((t + u) + (u2 + e2l)) + ((qx + qy) + qz);
+    // 1 / r: MUFU estimate y0 and the residual res = 1 - r^2 y0^2 in double-float; then
+    // 1/r = y0 (1 - res)^(-1/2) = y0 (1 + res/2 + 3 res^2/8 + ...), |res| < 2^-21
+    const float y0 = rsqrtf(S2);
+    const float q = __fmul_rn(y0, y0), qe = fmaf(y0, y0, -q);
+    const float pp = __fmul_rn(S2, q), pe = fmaf(S2, q, -pp);
+    const float res = ((1.f - pp) - pe) - fmaf(S2, qe, lo * q);
+    const float c = y0 * res * fmaf(0.375f, res, 0.5f);
+    // m / r = (m_h + m_l)(y0 + c)
+    w = __fmul_rn(mh, y0);
+    we = fmaf(mh, y0, -w) + fmaf(mh, c, ml * y0);
+}
+
 }  // namespace df
 }  // namespace frost

@@ -1973,6 +1973,31 @@ frost_status frost_energy_clusters(frost_ctx *c, double *E_kin, double *E_pot, d
     return FROST_OK;
 }
 
+// phi of every particle from all pairs and the energy reduction
+static void potential_all_pairs(frost_ctx *c)
+{
+    // the potential pass skips the tiles below each i-block's diagonal, so its blocks differ in
+    // work: eight waves of blocks (of its own occupancy) keep the last ones short
+    SplitShape sh;
+    {
+        const long long cap = (long long)potential_blocks_per_sm() * c->n_sm;
+        const int tiles = (int)((c->N + PAIR_TJ - 1) / PAIR_TJ);
+        sh.nblk_i = (int)((c->N + PAIR_BS - 1) / PAIR_BS);
+        const int ns = (int)std::min<long long>(tiles, std::max<long long>(1, (8 * cap + sh.nblk_i - 1) / sh.nblk_i));
+        sh.j_per_split = ((tiles + ns - 1) / ns) * PAIR_TJ;
+        sh.nsplit = (int)((c->N + sh.j_per_split - 1) / sh.j_per_split);
+    }
+    while ((size_t)sh.nsplit * c->N > c->part_elems && sh.nsplit > 1) {
+        const int tiles = (c->N + PAIR_TJ - 1) / PAIR_TJ;
+        const int ns = std::max(1, sh.nsplit / 2);
+        sh.j_per_split = ((tiles + ns - 1) / ns) * PAIR_TJ;
+        sh.nsplit = (c->N + sh.j_per_split - 1) / sh.j_per_split;
+    }
+    launch_potential(c->stream, c->x, c->m, c->N, c->eps2, (float4 *)c->recA, c->part, sh);
+    launch_energy_reduce(c->stream, c->x, c->v, c->m, c->N, c->part, sh.nsplit, c->dmisc->eres);
+    c->st.kernel_launches += 3;
+}
+
 frost_status frost_energy_momentum(frost_ctx *c, double *E_kin, double *E_pot, double P[3], double L[3])
 {
     if (!c) return fail(FROST_EINVAL, "NULL context");
@@ -1996,26 +2021,17 @@ frost_status frost_energy_momentum(frost_ctx *c, double *E_kin, double *E_pot, d
         }
         return FROST_OK;
     }
-    // the potential pass skips the tiles below each i-block's diagonal, so its blocks differ in
-    // work: eight waves of blocks (of its own occupancy) keep the last ones short
-    SplitShape sh;
-    {
-        const long long cap = (long long)potential_blocks_per_sm() * c->n_sm;
-        const int tiles = (int)((c->N + PAIR_TJ - 1) / PAIR_TJ);
-        sh.nblk_i = (int)((c->N + PAIR_BS - 1) / PAIR_BS);
-        const int ns = (int)std::min<long long>(tiles, std::max<long long>(1, (8 * cap + sh.nblk_i - 1) / sh.nblk_i));
-        sh.j_per_split = ((tiles + ns - 1) / ns) * PAIR_TJ;
-        sh.nsplit = (int)((c->N + sh.j_per_split - 1) / sh.j_per_split);
+    if (use_order(c, c->N)) {
+        const int ns = potential_tile_splits(c->N, c->n_sm, c->part_elems);
+        order_list(c, nullptr, c->N, c->opos, c->olist);
+        launch_tile_pack_pos(c->stream, c->olist, c->N, c->x, nullptr, 0.0, c->m, c->N, c->recA);
+        launch_pack_pot(c->stream, c->olist, c->x, c->m, c->N, (float4 *)c->recB);
+        launch_potential_tile(c->stream, c->olist, c->recA, (const float4 *)c->recB, c->N, c->eps2, ns, c->part);
+        launch_energy_reduce(c->stream, c->x, c->v, c->m, c->N, c->part, ns, c->dmisc->eres);
+        c->st.kernel_launches += 4;
+    } else {
+        potential_all_pairs(c);
     }
-    while ((size_t)sh.nsplit * c->N > c->part_elems && sh.nsplit > 1) {
-        const int tiles = (c->N + PAIR_TJ - 1) / PAIR_TJ;
-        const int ns = std::max(1, sh.nsplit / 2);
-        sh.j_per_split = ((tiles + ns - 1) / ns) * PAIR_TJ;
-        sh.nsplit = (c->N + sh.j_per_split - 1) / sh.j_per_split;
-    }
-    launch_potential(c->stream, c->x, c->m, c->N, c->eps2, (float4 *)c->recA, c->part, sh);
-    launch_energy_reduce(c->stream, c->x, c->v, c->m, c->N, c->part, sh.nsplit, c->dmisc->eres);
-    c->st.kernel_launches += 3;
     FROST_CUDA(cudaGetLastError());
     FROST_TRY(sync_misc(c));
     const double *e = c->hmisc->eres;

@@ -196,6 +196,8 @@ void launch_check_mass(cudaStream_t s, const double *m, int n, int *err);
 // launch_energy_reduce); rec: scratch of 48 B per particle
 void launch_potential(cudaStream_t s, const double *x, const double *m, int n, double eps2, float4 *rec,
                       double *part, const SplitShape &shape);
+// its records of a list (NULL: the identity) of all n particles
+void launch_pack_pot(cudaStream_t s, const int32_t *list, const double *x, const double *m, int n, float4 *rec);
 // blocks of the potential pass per SM (its occupancy)
 int potential_blocks_per_sm();
 // out[0] = T, out[1] = sum_i m_i phi_i, out[2..4] = P, out[5..7] = L (one block, fixed order)
@@ -301,6 +303,12 @@ void launch_tile_pack_grad(cudaStream_t s, const int32_t *list, int n, const dou
 void launch_wmax_tile(cudaStream_t s, const TileArgs &a, int n_sm, float *wmax);
 void launch_acc_tile(cudaStream_t s, const TileArgs &a, const float *wmax);
 void launch_grad_tile(cudaStream_t s, const TileArgs &a, const float *wmax);
+
+// phi as launch_potential for all n particles in the spatial order `list`: part[split][particle];
+// rec: position records (launch_tile_pack_pos), abs: records of launch_pack_pot
+int potential_tile_splits(int n, int n_sm, size_t part_elems);
+void launch_potential_tile(cudaStream_t s, const int32_t *list, const void *rec, const float4 *abs, int n, double eps2,
+                           int nsplit, double *part);
 
 // ---- single-CTA subtree solver (subtree.cu) ------------------------------------------
 constexpr int SUBTREE_MAX_FRAMES = 64;  // recursion frames per block (max_depth < 64)

@@ -101,3 +101,16 @@ def test_tiled_force_passes_of_two_lists(na, nb):
     one = f.accel_gradient(a, b, eps_grad=0.05)
     for key in ("acc", "acc_tilde", "grad"):
         assert torch.equal(one[key], out[key + "_a"]), key
+
+
+@pytest.mark.parametrize("n,masses,eps", [(16384, "equal", 0.0), (16449, "kroupa", 1e-3), (16447, "binaries", 0.0)])
+def test_tiled_potential_matches_the_all_pairs_sum(n, masses, eps):
+    # the FP64 mode's contexts sum all pairs from three-part positions; both are good to about
+    # 1e-13 a term
+    m, x, v = (ics.plummer_kroupa_binaries(n, 23) if masses == "binaries"
+               else ics.plummer(n, 23, ics.kroupa_masses(n, 23) if masses == "kroupa" else None))
+    x = x + np.array([3.0, -2.0, 1.0])
+    e = _frost(m, x, v, eps_soft=eps).energy()
+    r = _frost(m, x, v, eps_soft=eps, precision="fp64").energy()
+    assert abs(e["U"] / r["U"] - 1) < 1e-13
+    assert e["T"] == r["T"] and np.array_equal(e["P"], r["P"]) and np.array_equal(e["L"], r["L"])
