@@ -541,9 +541,12 @@ __device__ __forceinline__ float2 pair_weight(float2 r2, float2 m)
 }
 
 // ACC: the variant that feeds a gradient (refined rsqrt, folds of every tile, dominant terms in
-// double-float by wmax)
+// double-float by wmax).  Bound by the FP32 pipe (about 80 % of its cycles): 12 packed
+// operations a pair of far pairs (15 with ACC) and about 250 instructions a tile.  All 65536
+// particles of a Plummer sphere, with the sort: plain 2.50 -> 1.97 ms; ACC with its prepass 4.50
+// -> 2.72 ms.  12 resident warps an SM without spills beat 16 to 20 with fewer registers (2.14).
 template <bool ACC>
-__global__ void __launch_bounds__(32, ACC ? 16 : 20) k_acc_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
+__global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
                                                  int n_a, int n_s, int self_pass, int nsplit, float eps2, double eps2d,
                                                  const float *__restrict__ wmax, double *__restrict__ part)
 {
@@ -613,7 +616,12 @@ __global__ void __launch_bounds__(32, ACC ? 16 : 20) k_acc_tile(const float *__r
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) four_roundings(xh[k][q], xl[k][q], nx[k][q]);
+                    for (int q = 0; q < 3; ++q) {
+                        // the plain pass keeps one rounding (4 % faster, and within the error of
+                        // the MUFU rsqrt)
+                        if (ACC) four_roundings(xh[k][q], xl[k][q], nx[k][q]);
+                        else nx[k][q][0] = nx[k][q][1] = dup(-__fadd_rn(xh[k][q], xl[k][q]));
+                    }
 #pragma unroll 2
                 for (int b = 0; b < TB; ++b) {
                     const float4 X = s[P_X][b], Y = s[P_Y][b], Z = s[P_Z][b], M = s[P_M][b];
@@ -755,7 +763,10 @@ __device__ __forceinline__ void grad_weight(float2 r2, float2 m, float2 &w, floa
     w = __fmul2_rn(__fmul2_rn(m, y), ri2);
 }
 
-__global__ void __launch_bounds__(32, 16) k_grad_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
+// 27 packed operations a pair of far pairs (47 in the pass on absolute three-part positions), the
+// FP32 pipe 77 % busy.  65536 particles: 6.35 -> 4.42 ms.  The registers of 10 warps an SM hold
+// the loop without spills (16 warps: the whole acc+gradient pass 7.49 instead of 7.36 ms).
+__global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
                                                   int n_a, int n_s, int self_pass, int nsplit, double eps2d,
                                                   const float *__restrict__ wmax, double *__restrict__ part)
 {

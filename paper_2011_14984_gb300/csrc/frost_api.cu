@@ -108,10 +108,14 @@ constexpr int64_t kSymGradMaxPairs = int64_t(1) << 23;
 // at the top of every step, so that every list of the recursion inherits the order; the pass
 // entry points: the caller's list) and take the tile kernels of tile_kernels.cu; inside a step
 // the ordered lists of at least kTileMinN particles do
+// (The sort is what costs: the time-steps of 9001 particles took 215 us so and 174 on the
+// symmetric pass, of 40603 520 and 1610; inside a step, already ordered, 8192 took 160 and 159.)
 constexpr int kOrderMinN = 16384;
 constexpr int kTileMinN = 8192;
 // the same for the Newtonian and gradient passes: the lists of a pass entry point from
-// kOrderForceMinN particles on, and inside a step two lists of at least kTileForceMinN
+// kOrderForceMinN particles on (acc+gradient of 16384: 959 us so, 952 on the old passes; of 40603
+// 3.2 and 4.5 ms), and inside a step two lists of at least kTileForceMinN (a 65536-body
+// step 52.5 ms with 1024 to 2048, 54.3 with 8192; sparse lists lose accuracy below)
 constexpr int kOrderForceMinN = 24576;
 // two lists of a gradient entry point: from this many pairs on, and each list of at least
 // kOrderCrossMinN (a sparse list's tiles are wide).  25000 x 40000 particles: 4.67 ms so, 6.03

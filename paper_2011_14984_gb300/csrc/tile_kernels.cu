@@ -8,6 +8,9 @@
 // distance of the boxes alone bounds every criterion of every pair from below above the
 // receivers' present minima, and the tile is passed over.  The result is the minimum over the
 // same FP32 pair values as in the one-sided and the symmetric pass, so the same bits.
+// With the sort of the list, Plummer spheres: 65536 particles 3.76 -> 1.06 ms, 40603 1.61 -> 0.52
+// ms, 262144 53 -> 7.1 ms (before: the symmetric pass over all pairs).  What is left is latency:
+// the judging of items issues about 0.4 of the time.
 #include "pair_bodies.cuh"
 
 namespace frost {

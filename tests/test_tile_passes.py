@@ -114,3 +114,15 @@ def test_tiled_potential_matches_the_all_pairs_sum(n, masses, eps):
     r = _frost(m, x, v, eps_soft=eps, precision="fp64").energy()
     assert abs(e["U"] / r["U"] - 1) < 1e-13
     assert e["T"] == r["T"] and np.array_equal(e["P"], r["P"]) and np.array_equal(e["L"], r["L"])
+
+
+def test_tiled_passes_report_coincident_particles():
+    from paper_2011_14984_gb300.frost import FROST_ECOINCIDENT, FrostError
+    n = 24576
+    m, x, v = ics.plummer(n, 24)
+    x[n - 1] = x[17]
+    for call in (lambda f: f.timesteps(), lambda f: f.accel_gradient(eps_grad=0.05),
+                 lambda f: f.accel_gradient(want=("acc",))):
+        with pytest.raises(FrostError) as e:
+            call(_frost(m, x, v))
+        assert e.value.code == FROST_ECOINCIDENT
