@@ -221,7 +221,9 @@ frost_status frost_accel_pairwise(frost_ctx *ctx, const int32_t *a, int64_t n_a,
  * its dominant terms (above 1/16 of its max m / r^3) out of the FP32 sums and evaluates them
  * in double-float, as frost_accel_gradient does, with no limit on their number for the set
  * summed by the reduction; sums are in a fixed order, so results are deterministic.  With
- * frost_opts.sym_cross = -1, and in FP64 mode, two one-sided passes per kind.  a, b: device
+ * frost_opts.sym_cross = -1, in FP64 mode, and with sym_cross = 0 for two lists of at least
+ * 8192 particles each and 2^27 pairs: two one-sided passes per kind, the accelerations and
+ * gradients of a having the bits of frost_accel_gradient(a, b).  a, b: device
  * int32 lists (or NULL = identity) of n_a and n_b indices with no index in both (else
  * FROST_EINVAL); outputs: device [n][3] doubles, each may be NULL.  Softened like
  * frost_accel_gradient.  Accuracy: as frost_accel_gradient.  Synchronises.

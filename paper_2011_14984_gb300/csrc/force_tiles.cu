@@ -1,4 +1,4 @@
-// Mixed-precision Newtonian and gradient passes of spatially ordered lists, tile by tile
+// Mixed-precision Newtonian and gradient passes of a spatially ordered list, tile by tile
 // (sm_103a).  A warp takes 64 receivers (two a lane) against its share of the sources' tiles of
 // 64 and treats a tile by the distance of its box from the receivers' box.
 //
@@ -338,17 +338,16 @@ __device__ __forceinline__ void wmax_tile(const Group &W, int g, const float *__
     }
 }
 
-__global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
-                                                  int n_a, int n_s, int self_pass, int nsplit, float eps2,
+__global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ rec, int n, int nsplit, float eps2,
                                                   float *__restrict__ wmax)
 {
     __shared__ float4 s[7][TB];
     __shared__ Group W;
-    const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n_s + TJ - 1) / TJ;
-    const Head *jh = heads(jrec, n_s, P_ROWS);
-    load_group(W, irec, n_a, P_ROWS, P_XL, g);
+    const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n + TJ - 1) / TJ;
+    const Head *jh = heads(rec, n, P_ROWS);
+    load_group(W, rec, n, P_ROWS, P_XL, g);
     float q[2] = {INFINITY, INFINITY};
-    // first the tile whose centre is nearest (in a self pass the receivers' own)
+    // first the tile whose centre is nearest (the receivers' own, if it is in this split)
     float best = INFINITY;
     int first = -1;
     for (int t = blockIdx.y + lane * nsplit; t < ntiles; t += 32 * nsplit) {
@@ -365,14 +364,14 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
         const unsigned mask = __ballot_sync(kFull, best == d && first >= 0);
         if (!mask) return;
         first = __shfl_sync(kFull, first, __ffs(mask) - 1);
-        wmax_tile(W, g, jrec, jh[first], first, self_pass && first == g, eps2, s, q);
+        wmax_tile(W, g, rec, jh[first], first, first == g, eps2, s, q);
     }
     // then those that can still hold a larger m_j / r^3 for some receiver: box against box, then
     // every receiver against the box (a few receivers far from the others stretch the group's box
     // and bound, and it would look into 11 instead of 1 % of a 65536-body sphere's tiles)
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
         const int t = t0 + lane * nsplit;
-        const float qmax = 1.0001f * warp_max(fmaxf(g * TJ + slot_of(0) < n_a ? q[0] : 0.f, g * TJ + slot_of(1) < n_a ? q[1] : 0.f));
+        const float qmax = 1.0001f * warp_max(fmaxf(g * TJ + slot_of(0) < n ? q[0] : 0.f, g * TJ + slot_of(1) < n ? q[1] : 0.f));
         bool near = false;
         if (t < ntiles && t != first) {
             const float4 c = jh[t].c, h = jh[t].h;
@@ -384,8 +383,8 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
             bool any = false;
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                any = any || (g * TJ + slot_of(k) < n_a && !((point_gap2(W, k, J.c, J.h) + eps2) * J.h.w > 1.0001f * q[k]));
-            if (__any_sync(kFull, any)) wmax_tile(W, g, jrec, J, tt, self_pass && tt == g, eps2, s, q);
+                any = any || (g * TJ + slot_of(k) < n && !((point_gap2(W, k, J.c, J.h) + eps2) * J.h.w > 1.0001f * q[k]));
+            if (__any_sync(kFull, any)) wmax_tile(W, g, rec, J, tt, tt == g, eps2, s, q);
         }
     }
 #pragma unroll
@@ -393,7 +392,7 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ irec
         const float y = rsqrtf(q[k]);
         // non-negative floats order as their bit patterns
         const int i = g * TJ + slot_of(k);
-        if (i < n_a) atomicMax((int *)&wmax[i], __float_as_int(y * y * y));
+        if (i < n) atomicMax((int *)&wmax[i], __float_as_int(y * y * y));
     }
 }
 
@@ -484,19 +483,18 @@ __device__ __forceinline__ df::dfloat tile_sep(float jc, float jh, float jl, flo
 }
 
 // evaluates the slots of a lane's receiver k (n of them)
-__device__ __noinline__ void acc_flush(Slots &S, const float *__restrict__ irec, const Head *__restrict__ ih,
-                                       const float *__restrict__ jrec, const Head *__restrict__ jh, int i, int k, int n,
-                                       double eps2d)
+__device__ __noinline__ void acc_flush(Slots &S, const float *__restrict__ rec, const Head *__restrict__ hd, int i, int k,
+                                       int n, double eps2d)
 {
     if (n == 0) return;
-    const float *ti = irec + (size_t)(i / TJ) * P_ROWS * TJ + i % TJ;
-    const float4 ci = ih[i / TJ].c;
+    const float *ti = rec + (size_t)(i / TJ) * P_ROWS * TJ + i % TJ;
+    const float4 ci = hd[i / TJ].c;
     using df::dfloat;
     const dfloat e2 = df::from_double(eps2d);
     for (int s = 0; s < n; ++s) {
         const int j = S.j[k][s];
-        const float *t = jrec + (size_t)(j / TJ) * P_ROWS * TJ + j % TJ;
-        const float4 c = jh[j / TJ].c;
+        const float *t = rec + (size_t)(j / TJ) * P_ROWS * TJ + j % TJ;
+        const float4 c = hd[j / TJ].c;
         const dfloat dx = tile_sep(c.x, t[P_X * TJ], t[P_XL * TJ], ci.x, ti[P_X * TJ], ti[P_XL * TJ]);
         const dfloat dy = tile_sep(c.y, t[P_Y * TJ], t[P_YL * TJ], ci.y, ti[P_Y * TJ], ti[P_YL * TJ]);
         const dfloat dz = tile_sep(c.z, t[P_Z * TJ], t[P_ZL * TJ], ci.z, ti[P_Z * TJ], ti[P_ZL * TJ]);
@@ -546,22 +544,23 @@ __device__ __forceinline__ float2 pair_weight(float2 r2, float2 m)
 // particles of a Plummer sphere, with the sort: plain 2.50 -> 1.97 ms; ACC with its prepass 4.50
 // -> 2.72 ms.  12 resident warps an SM without spills beat 16 to 20 with fewer registers (2.14).
 template <bool ACC>
-__global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
-                                                 int n_a, int n_s, int self_pass, int nsplit, float eps2, double eps2d,
-                                                 const float *__restrict__ wmax, double *__restrict__ part)
+__global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__restrict__ rec, int n, int nsplit,
+                                                                      float eps2, double eps2d,
+                                                                      const float *__restrict__ wmax,
+                                                                      double *__restrict__ part)
 {
     __shared__ float4 s[8][TB];
     __shared__ Group W;
     Slots S;
-    const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n_s + TJ - 1) / TJ;
-    const Head *ih = heads(irec, n_a, P_ROWS), *jh = heads(jrec, n_s, P_ROWS);
-    load_group(W, irec, n_a, P_ROWS, P_XL, g);
+    const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n + TJ - 1) / TJ;
+    const Head *jh = heads(rec, n, P_ROWS);
+    load_group(W, rec, n, P_ROWS, P_XL, g);
     float thr[2] = {INFINITY, INFINITY}, qk[2] = {0.f, 0.f}, qthr = 0.f;
     int cnt[2] = {0, 0};
     if (ACC) {
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if (g * TJ + slot_of(k) < n_a) thr[k] = SLOT_FRACTION * wmax[g * TJ + slot_of(k)];
+            if (g * TJ + slot_of(k) < n) thr[k] = SLOT_FRACTION * wmax[g * TJ + slot_of(k)];
         // r^2 m^(-2/3) at the threshold: a pair above it is below the threshold
 #pragma unroll
         for (int k = 0; k < 2; ++k) qk[k] = 1.0001f * exp2f(-0.6666667f * log2f(thr[k]));
@@ -571,13 +570,13 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
     const float2 e2 = dup(eps2);
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
         unsigned fm, nm;
-        judge_tiles<ACC>(W, jh, ntiles, t0, nsplit, self_pass ? g : -1, g * TJ + slot_of(0) < n_a, g * TJ + slot_of(1) < n_a, qthr,
+        judge_tiles<ACC>(W, jh, ntiles, t0, nsplit, g, g * TJ + slot_of(0) < n, g * TJ + slot_of(1) < n, qthr,
                          qk, fm, nm);
         // the next tile's rows wait in registers: 64 pieces of the far rows, 128 of all
         auto next_bit = [&]() { return fm ? __ffs(fm) - 1 : __ffs(nm) - 1; };
         float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
         auto fetch = [&]() {
-            const float4 *tr = (const float4 *)(jrec + (size_t)(t0 + next_bit() * nsplit) * P_ROWS * TJ);
+            const float4 *tr = (const float4 *)(rec + (size_t)(t0 + next_bit() * nsplit) * P_ROWS * TJ);
             n0 = tr[lane];
             n1 = tr[32 + lane];
             if (!fm) {
@@ -640,7 +639,7 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                         }
                 }
             } else {
-                const bool diag = self_pass && t == g;
+                const bool diag = t == g;
 #pragma unroll 1
                 for (int b = 0; b < TB; ++b) {
                     const float4 X = s[P_X][b], Y = s[P_Y][b], Z = s[P_Z][b], M = s[P_M][b];
@@ -688,13 +687,13 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int r = slot_of(k);
-        if (ACC) acc_flush(S, irec, ih, jrec, jh, g * TJ + slot_of(k), k, cnt[k], eps2d);
-        if (g * TJ + r >= n_a) continue;
-        double *p = part + (size_t)blockIdx.y * 3 * n_a + g * TJ + r;
+        if (ACC) acc_flush(S, rec, jh, g * TJ + slot_of(k), k, cnt[k], eps2d);
+        if (g * TJ + r >= n) continue;
+        double *p = part + (size_t)blockIdx.y * 3 * n + g * TJ + r;
         for (int q = 0; q < 3; ++q) {
             double v = group_total(W, q, r);
             if (ACC) v += slots_total(S, k, q);
-            p[(size_t)q * n_a] = v;
+            p[(size_t)q * n] = v;
         }
     }
 }
@@ -707,19 +706,18 @@ struct GroupA {
     float h[3][TJ], l[3][TJ];
 };
 
-__device__ __noinline__ void grad_flush(Slots &S, const float *__restrict__ irec, const Head *__restrict__ ih,
-                                        const float *__restrict__ jrec, const Head *__restrict__ jh, int i, int k, int n,
-                                        double eps2d)
+__device__ __noinline__ void grad_flush(Slots &S, const float *__restrict__ rec, const Head *__restrict__ hd, int i, int k,
+                                        int n, double eps2d)
 {
     if (n == 0) return;
-    const float *ti = irec + (size_t)(i / TJ) * G_ROWS * TJ + i % TJ;
-    const float4 ci = ih[i / TJ].c, ai = ih[i / TJ].a;
+    const float *ti = rec + (size_t)(i / TJ) * G_ROWS * TJ + i % TJ;
+    const float4 ci = hd[i / TJ].c, ai = hd[i / TJ].a;
     using df::dfloat;
     const dfloat e2 = df::from_double(eps2d);
     for (int s = 0; s < n; ++s) {
         const int j = S.j[k][s];
-        const float *t = jrec + (size_t)(j / TJ) * G_ROWS * TJ + j % TJ;
-        const float4 c = jh[j / TJ].c, a = jh[j / TJ].a;
+        const float *t = rec + (size_t)(j / TJ) * G_ROWS * TJ + j % TJ;
+        const float4 c = hd[j / TJ].c, a = hd[j / TJ].a;
         const dfloat dx = tile_sep(c.x, t[G_X * TJ], t[G_XL * TJ], ci.x, ti[G_X * TJ], ti[G_XL * TJ]);
         const dfloat dy = tile_sep(c.y, t[G_Y * TJ], t[G_YL * TJ], ci.y, ti[G_Y * TJ], ti[G_YL * TJ]);
         const dfloat dz = tile_sep(c.z, t[G_Z * TJ], t[G_ZL * TJ], ci.z, ti[G_Z * TJ], ti[G_ZL * TJ]);
@@ -766,29 +764,28 @@ __device__ __forceinline__ void grad_weight(float2 r2, float2 m, float2 &w, floa
 // 27 packed operations a pair of far pairs (47 in the pass on absolute three-part positions), the
 // FP32 pipe 77 % busy.  65536 particles: 6.35 -> 4.42 ms.  The registers of 10 warps an SM hold
 // the loop without spills (16 warps: the whole acc+gradient pass 7.49 instead of 7.36 ms).
-__global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ irec, const float *__restrict__ jrec,
-                                                  int n_a, int n_s, int self_pass, int nsplit, double eps2d,
-                                                  const float *__restrict__ wmax, double *__restrict__ part)
+__global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ rec, int n, int nsplit, double eps2d,
+                                                      const float *__restrict__ wmax, double *__restrict__ part)
 {
     __shared__ float4 s[G_ROWS][TB];
     __shared__ Group W;
     __shared__ GroupA A;
     Slots S;
-    const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n_s + TJ - 1) / TJ;
-    const Head *ih = heads(irec, n_a, G_ROWS), *jh = heads(jrec, n_s, G_ROWS);
-    load_group(W, irec, n_a, G_ROWS, G_XL, g);
+    const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n + TJ - 1) / TJ;
+    const Head *jh = heads(rec, n, G_ROWS);
+    load_group(W, rec, n, G_ROWS, G_XL, g);
 #pragma unroll
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            A.h[q][slot_of(k)] = irec[((size_t)g * G_ROWS + G_AX + q) * TJ + slot_of(k)];
-            A.l[q][slot_of(k)] = irec[((size_t)g * G_ROWS + G_AXL + q) * TJ + slot_of(k)];
+            A.h[q][slot_of(k)] = rec[((size_t)g * G_ROWS + G_AX + q) * TJ + slot_of(k)];
+            A.l[q][slot_of(k)] = rec[((size_t)g * G_ROWS + G_AXL + q) * TJ + slot_of(k)];
         }
     float thr[2] = {INFINITY, INFINITY};
     int cnt[2] = {0, 0};
 #pragma unroll
     for (int k = 0; k < 2; ++k)
-        if (g * TJ + slot_of(k) < n_a) thr[k] = SLOT_FRACTION * wmax[g * TJ + slot_of(k)];
+        if (g * TJ + slot_of(k) < n) thr[k] = SLOT_FRACTION * wmax[g * TJ + slot_of(k)];
     float qk[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) qk[k] = 1.0001f * exp2f(-0.6666667f * log2f(thr[k]));
@@ -797,13 +794,13 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
     const float2 e2 = dup((float)eps2d);
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
         unsigned fm, nm;
-        judge_tiles<true>(W, jh, ntiles, t0, nsplit, self_pass ? g : -1, g * TJ + slot_of(0) < n_a, g * TJ + slot_of(1) < n_a, qthr,
+        judge_tiles<true>(W, jh, ntiles, t0, nsplit, g, g * TJ + slot_of(0) < n, g * TJ + slot_of(1) < n, qthr,
                          qk, fm, nm);
         auto next_bit = [&]() { return fm ? __ffs(fm) - 1 : __ffs(nm) - 1; };
         // the next tile's far rows wait in registers, 112 of its 208 pieces
         float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
         auto fetch = [&]() {
-            const float4 *tr = (const float4 *)(jrec + (size_t)(t0 + next_bit() * nsplit) * G_ROWS * TJ);
+            const float4 *tr = (const float4 *)(rec + (size_t)(t0 + next_bit() * nsplit) * G_ROWS * TJ);
             n0 = tr[lane];
             n1 = tr[32 + lane];
             n2 = tr[64 + lane];
@@ -823,7 +820,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
             sf[64 + lane] = n2;
             sf[96 + lane] = n3;
             if (!isfar) {
-                const float4 *tr = (const float4 *)(jrec + (size_t)t * G_ROWS * TJ);
+                const float4 *tr = (const float4 *)(rec + (size_t)t * G_ROWS * TJ);
                 sf[128 + lane] = tr[128 + lane];
                 sf[160 + lane] = tr[160 + lane];
                 if (lane < 16) sf[192 + lane] = tr[192 + lane];
@@ -888,7 +885,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                         }
                 }
             } else {
-                const bool diag = self_pass && t == g;
+                const bool diag = t == g;
 #pragma unroll 1
                 for (int b = 0; b < TB; ++b) {
                     const float4 X = s[G_X][b], Y = s[G_Y][b], Z = s[G_Z][b], M = s[G_M][b];
@@ -942,11 +939,11 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int r = slot_of(k);
-        grad_flush(S, irec, ih, jrec, jh, g * TJ + slot_of(k), k, cnt[k], eps2d);
-        if (g * TJ + r >= n_a) continue;
-        double *p = part + (size_t)blockIdx.y * 3 * n_a + g * TJ + r;
+        grad_flush(S, rec, jh, g * TJ + slot_of(k), k, cnt[k], eps2d);
+        if (g * TJ + r >= n) continue;
+        double *p = part + (size_t)blockIdx.y * 3 * n + g * TJ + r;
         for (int q = 0; q < 3; ++q)
-            p[(size_t)q * n_a] = group_total(W, q, r) + slots_total(S, k, q);
+            p[(size_t)q * n] = group_total(W, q, r) + slots_total(S, k, q);
     }
 }
 
@@ -1057,14 +1054,14 @@ void launch_potential_tile(cudaStream_t s, const int32_t *list, const void *rec,
     k_potential_tile<<<dim3((n + TJ - 1) / TJ, nsplit), 32, 0, s>>>(list, (const float *)rec, abs, n, nsplit, eps2, part);
 }
 
-int tile_splits(int n_a, int n_s, int n_sm, size_t part_elems)
+int tile_splits(int n, int n_sm, size_t part_elems)
 {
-    const long long ngroups = (n_a + TJ - 1) / TJ, ntiles = (n_s + TJ - 1) / TJ;
+    const long long ntiles = (n + TJ - 1) / TJ;
     // eight rounds of about 20 resident warps an SM, each warp 16 tiles at least (its slots, a few
     // double-float terms a lane whatever it sees, cost as much as several tiles: with 4 tiles a
     // warp a 65536-body step took 55.4 ms, with 16 52.3), the partials within their buffer
-    long long ns = std::min((8LL * 20 * n_sm + ngroups - 1) / ngroups, (ntiles + 15) / 16);
-    ns = std::min<long long>(ns, (long long)(part_elems / (3 * (size_t)n_a)));
+    long long ns = std::min((8LL * 20 * n_sm + ntiles - 1) / ntiles, (ntiles + 15) / 16);
+    ns = std::min<long long>(ns, (long long)(part_elems / (3 * (size_t)n)));
     return (int)std::max<long long>(1, ns);
 }
 
@@ -1085,29 +1082,25 @@ void launch_tile_pack_grad(cudaStream_t s, const int32_t *list, int n, const dou
 
 void launch_wmax_tile(cudaStream_t s, const TileArgs &a, int n_sm, float *wmax)
 {
-    cudaMemsetAsync(wmax, 0, sizeof(float) * a.n_a, s);
-    const int ngroups = (a.n_a + TJ - 1) / TJ, ntiles = (a.n_s + TJ - 1) / TJ;
+    cudaMemsetAsync(wmax, 0, sizeof(float) * a.n, s);
+    const int ntiles = (a.n + TJ - 1) / TJ;
     // few tiles are looked into, so a group is split only to fill the SMs
-    const int ns = std::max(1, std::min((ntiles + 31) / 32, (16 * n_sm + ngroups - 1) / ngroups));
-    k_wmax_tile<<<dim3(ngroups, ns), 32, 0, s>>>((const float *)a.irec, (const float *)a.jrec, a.n_a, a.n_s, a.self_pass,
-                                                 ns, (float)a.eps2, wmax);
+    const int ns = std::max(1, std::min((ntiles + 31) / 32, (16 * n_sm + ntiles - 1) / ntiles));
+    k_wmax_tile<<<dim3(ntiles, ns), 32, 0, s>>>((const float *)a.rec, a.n, ns, (float)a.eps2, wmax);
 }
 
 void launch_acc_tile(cudaStream_t s, const TileArgs &a, const float *wmax)
 {
-    const dim3 grid((a.n_a + TJ - 1) / TJ, a.nsplit);
+    const dim3 grid((a.n + TJ - 1) / TJ, a.nsplit);
     if (wmax)
-        k_acc_tile<true><<<grid, 32, 0, s>>>((const float *)a.irec, (const float *)a.jrec, a.n_a, a.n_s, a.self_pass,
-                                             a.nsplit, (float)a.eps2, a.eps2, wmax, a.part);
+        k_acc_tile<true><<<grid, 32, 0, s>>>((const float *)a.rec, a.n, a.nsplit, (float)a.eps2, a.eps2, wmax, a.part);
     else
-        k_acc_tile<false><<<grid, 32, 0, s>>>((const float *)a.irec, (const float *)a.jrec, a.n_a, a.n_s, a.self_pass,
-                                              a.nsplit, (float)a.eps2, a.eps2, nullptr, a.part);
+        k_acc_tile<false><<<grid, 32, 0, s>>>((const float *)a.rec, a.n, a.nsplit, (float)a.eps2, a.eps2, nullptr, a.part);
 }
 
 void launch_grad_tile(cudaStream_t s, const TileArgs &a, const float *wmax)
 {
-    k_grad_tile<<<dim3((a.n_a + TJ - 1) / TJ, a.nsplit), 32, 0, s>>>((const float *)a.irec, (const float *)a.jrec, a.n_a,
-                                                                 a.n_s, a.self_pass, a.nsplit, a.eps2, wmax, a.part);
+    k_grad_tile<<<dim3((a.n + TJ - 1) / TJ, a.nsplit), 32, 0, s>>>((const float *)a.rec, a.n, a.nsplit, a.eps2, wmax, a.part);
 }
 
 }  // namespace frost

@@ -104,6 +104,14 @@ constexpr int64_t kSymCrossPrepassMinPairs = int64_t(1) << 26;
 // B-side reduction and dominant-term ballots cost what the saved pair bodies save)
 constexpr int64_t kSymGradMaxPairs = int64_t(1) << 23;
 
+// the pairwise gradient entry point takes two one-sided passes per kind (the bits of
+// frost_accel_gradient's) for two lists of at least this size and this many pairs: 25000 x 40000
+// particles, a halo around its core, 5.96 ms so and 6.25 on the symmetric kernels, 12001 x 11905
+// 1.23 and 1.55, 65536 x 32768 12.2 and 13.0 (lists mixed at random: 5.79 and 5.75, 1.22 and
+// 1.34, 11.9 and 11.7)
+constexpr int64_t kOneSidedPairwiseMinPairs = int64_t(1) << 27;
+constexpr int kOneSidedPairwiseMinN = 8192;
+
 // mixed mode: sets from this size on are put in spatial order (a frost_step call: all particles
 // at the top of every step, so that every list of the recursion inherits the order; the pass
 // entry points: the caller's list) and take the tile kernels of tile_kernels.cu; inside a step
@@ -112,17 +120,13 @@ constexpr int64_t kSymGradMaxPairs = int64_t(1) << 23;
 // symmetric pass, of 40603 520 and 1610; inside a step, already ordered, 8192 took 160 and 159.)
 constexpr int kOrderMinN = 16384;
 constexpr int kTileMinN = 8192;
-// the same for the Newtonian and gradient passes: the lists of a pass entry point from
+// the same for the Newtonian and gradient passes of one list: a pass entry point's from
 // kOrderForceMinN particles on (acc+gradient of 16384: 959 us so, 952 on the old passes; of 40603
-// 3.2 and 4.5 ms), and inside a step two lists of at least kTileForceMinN (a 65536-body
-// step 52.5 ms with 1024 to 2048, 54.3 with 8192; sparse lists lose accuracy below)
+// 3.2 and 4.5 ms), and inside a step lists of at least kTileForceMinN.  Passes between two lists
+// do not take the tiles: a list's dominant terms then sit in few tiles of the other, and with
+// slots enough to keep its gradient as good as on the old passes (64 a split) the tiles are no
+// faster (25000 x 40000 particles 8.3 against 6.3 ms).
 constexpr int kOrderForceMinN = 24576;
-// two lists of a gradient entry point: from this many pairs on, and each list of at least
-// kOrderCrossMinN (a sparse list's tiles are wide).  25000 x 40000 particles: 4.67 ms so, 6.03
-// on the symmetric passes; 12001 x 11905: 1.37 and 1.46; 16717 x 6101: 1.14 and 1.16; 2049 x
-// 65537: 1.32 and 1.35, but with errors a quarter larger
-constexpr int64_t kOrderCrossMinPairs = int64_t(1) << 27;
-constexpr int kOrderCrossMinN = 8192;
 constexpr int kTileForceMinN = 4096;
 
 // autotuner rows: the pass kinds, and the Newtonian pass that feeds a gradient (mixed mode:
@@ -453,25 +457,16 @@ void order_list(frost_ctx *c, const int32_t *list, int n, int32_t *pos, int32_t 
 // |a| of a tile fails for most of them (20 against 7 ms at 65536 particles)
 bool tile_tstep(const frost_ctx *c, int n) { return c->ordered && n >= kTileMinN && !(c->sym & FROST_FLYBY_EXACT); }
 
-// whether the Newtonian and gradient passes between two lists (or of one) of the running call take
-// the tile kernels
-bool tile_force(const frost_ctx *c, int nA, int nB) { return c->ordered && std::min(nA, nB) >= kTileForceMinN; }
+// whether the Newtonian and gradient passes of a list of the running call take the tile kernels
+bool tile_force(const frost_ctx *c, int n) { return c->ordered && n >= kTileForceMinN; }
 
-bool order_cross(const frost_ctx *c, int nA, int nB)
-{
-    return c->ord && std::min(nA, nB) >= kOrderCrossMinN && (int64_t)nA * nB >= kOrderCrossMinPairs;
-}
-
-TileArgs tile_args(const frost_ctx *c, const Lane &L, const void *irec, int nA, const void *jrec, int nB, bool self)
+TileArgs tile_args(const frost_ctx *c, const Lane &L, const void *rec, int n)
 {
     TileArgs a;
-    a.irec = irec;
-    a.jrec = jrec;
-    a.n_a = nA;
-    a.n_s = nB;
-    a.self_pass = self ? 1 : 0;
+    a.rec = rec;
+    a.n = n;
     a.eps2 = c->eps2;
-    a.nsplit = tile_splits(nA, nB, c->n_sm, c->part_elems);
+    a.nsplit = tile_splits(n, c->n_sm, c->part_elems);
     a.part = L.part;
     return a;
 }
@@ -482,8 +477,8 @@ TileArgs tile_args(const frost_ctx *c, const Lane &L, const void *irec, int nA, 
 // With hist (mixed mode, with wmax): the |a| histogram of the pass is added to hist (zeroed by
 // the caller) for the hot-source classification of mark_hot.  kick: the kick of A by the
 // result, fused into the finalisation.  irec / jrec: records already packed by the caller
-// (NULL: packed here into the lane's recA / recB).  tile: the lists are in spatial order and
-// take the tile kernels (packed records are theirs); omap: the rows of out_aos.
+// (NULL: packed here into the lane's recA / recB).  tile (self only): the list is in spatial order
+// and takes the tile kernels (packed records are theirs); omap: the rows of out_aos.
 bool use_sym_self(const frost_ctx *c, int n) { return c->sym_cross > 0 || (c->sym_cross == 0 && n >= kSymTstepMinN); }
 
 void pass_acc(frost_ctx *c, Lane &L, const int32_t *A, int nA, const int32_t *B, int nB, bool self,
@@ -508,10 +503,9 @@ void pass_acc(frost_ctx *c, Lane &L, const int32_t *A, int nA, const int32_t *B,
     if (tile) {
         if (!irec) {
             launch_tile_pack_pos(L.s, A, nA, c->x, nullptr, 0.0, c->m, c->N, L.recA);
-            if (!self) launch_tile_pack_pos(L.s, B, nB, c->x, nullptr, 0.0, c->m, c->N, L.recB);
-            c->st.kernel_launches += self ? 1 : 2;
+            c->st.kernel_launches += 1;
         }
-        const TileArgs t = tile_args(c, L, irec ? irec : L.recA, nA, irec ? jrec : (self ? L.recA : L.recB), nB, self);
+        const TileArgs t = tile_args(c, L, irec ? irec : L.recA, nA);
         {
             TimedScope ts(c, L.s, PASS_ACC, pairs);
             if (accurate) launch_wmax_tile(L.s, t, c->n_sm, wmax);
@@ -612,8 +606,7 @@ void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA
     if (irec) {
         // packed by the caller
     } else if (tile) {
-        launch_tile_pack_grad(L.s, A, nA, c->x, c->m, c->N, aA, self ? hotB : nullptr, L.recA);
-        if (!self) launch_tile_pack_grad(L.s, B, nB, c->x, c->m, c->N, aB, hotB, L.recB);
+        launch_tile_pack_grad(L.s, A, nA, c->x, c->m, c->N, aA, hotB, L.recA);
     } else if (c->mixed) {
         // hot sources: masses zeroed in the FP32 source records, their terms summed in
         // double-float by k_grad_hot
@@ -628,7 +621,7 @@ void pass_grad(frost_ctx *c, Lane &L, const int32_t *A, int nA, const double *aA
     const int64_t pairs = self ? (int64_t)nA * (nA - 1) : (int64_t)nA * nB;
     int nsplit;
     if (tile) {
-        const TileArgs t = tile_args(c, L, ir, nA, jr, nB, self);
+        const TileArgs t = tile_args(c, L, ir, nA);
         nsplit = t.nsplit;
         TimedScope ts(c, L.s, PASS_GRAD, pairs);
         launch_grad_tile(L.s, t, wmax);
@@ -754,53 +747,20 @@ void drift_pack(frost_ctx *c, Lane &L, const int32_t *list, int n, double dt, vo
 }
 
 // position records of the list for a Newtonian pass (both variants read the same records)
-void pack_acc(frost_ctx *c, Lane &L, const int32_t *list, int n, void *rec, bool tile = false)
+void pack_acc(frost_ctx *c, Lane &L, const int32_t *list, int n, void *rec)
 {
     if (n <= 0) return;
-    if (tile) {
-        launch_tile_pack_pos(L.s, list, n, c->x, nullptr, 0.0, c->m, c->N, rec);
-        c->st.kernel_launches += 1;
-        return;
-    }
     pack_pos(c, L, list, n, rec);
 }
 
 // gradient records of the list with accelerations a ([3][n]); mixed mode: masses of the hot
 // particles (mask) zeroed, their terms are summed in double-float by k_grad_hot
-void pack_grad(frost_ctx *c, Lane &L, const int32_t *list, int n, const double *a, void *rec, const uint32_t *mask,
-               bool tile = false)
+void pack_grad(frost_ctx *c, Lane &L, const int32_t *list, int n, const double *a, void *rec, const uint32_t *mask)
 {
     if (n <= 0) return;
-    if (tile) launch_tile_pack_grad(L.s, list, n, c->x, c->m, c->N, a, mask, rec);
-    else if (c->mixed) launch_pack_grad_mixed(L.s, list, n, c->x, c->m, c->N, a, (float4 *)rec, mask);
+    if (c->mixed) launch_pack_grad_mixed(L.s, list, n, c->x, c->m, c->N, a, (float4 *)rec, mask);
     else launch_pack_grad_fp64(L.s, list, n, c->x, c->m, c->N, a, (double4_32a *)rec);
     c->st.kernel_launches += 1;
-}
-
-// The force-gradient kick of two disjoint lists due to each other on the tile kernels, both lists
-// put in spatial order first and the results in the callers' orders (any may be NULL; only_a:
-// without B's gradient).  The order's buffers are free outside a step.
-void grad_pairwise_tile(frost_ctx *c, Lane &M, const int32_t *A, int nA, const int32_t *B, int nB, double eps_grad,
-                        double *acc_a, double *acc_b, double *at_a, double *at_b, double *g_a, double *g_b, bool only_a)
-{
-    int32_t *SA = c->olist, *SB = c->ord;
-    const int32_t *pA = c->opos, *pB = c->ptmp;
-    order_list(c, A, nA, c->opos, SA);
-    order_list(c, B, nB, c->ptmp, SB);
-    unsigned *h = zero_hists(M);
-    pack_acc(c, M, SA, nA, M.recA, true);
-    pack_acc(c, M, SB, nB, M.recB, true);
-    pass_acc(c, M, SA, nA, SB, nB, false, M.aA, acc_a, M.wA, h, KickArgs(), M.recA, M.recB, false, true, pA);
-    pass_acc(c, M, SB, nB, SA, nA, false, M.aB, acc_b, M.wB, h + HOT_BINS, KickArgs(), M.recB, M.recA, false, true, pB);
-    mark_hot(c, M, nA, nB, false, M.aA, h, h + HOT_BINS, nB, M.hA);
-    mark_hot(c, M, nB, nA, false, M.aB, h + HOT_BINS, h, nA, M.hB);
-    pack_grad(c, M, SA, nA, M.aA, M.recA, M.hA, true);
-    pack_grad(c, M, SB, nB, M.aB, M.recB, M.hB, true);
-    pass_grad(c, M, SA, nA, M.aA, SB, nB, M.aB, false, eps_grad, nullptr, at_a, g_a, M.wA, M.hB, KickArgs(), M.recA,
-              M.recB, true, pA);
-    if (!only_a)
-        pass_grad(c, M, SB, nB, M.aB, SA, nA, M.aA, false, eps_grad, nullptr, at_b, g_b, M.wB, M.hA, KickArgs(), M.recB,
-                  M.recA, true, pB);
 }
 
 // Algorithm fsi on the set S with step dt.  Each kick is fused into the finalisation of the
@@ -813,7 +773,7 @@ void fsi(frost_ctx *c, Lane &L, const int32_t *S, int nS, double dt, int cache =
     if (nS <= 0) return;
     c->st.fsi_calls += 1;
     if (nS < 2) cache = 0;
-    const bool tile = tile_force(c, nS, nS);
+    const bool tile = tile_force(c, nS);
     if (cache == 2) {
         launch_kick_by_particle(L.s, S, nS, c->v, c->N, c->aC, dt / 6.0);
         c->st.kernel_launches += 1;
@@ -1001,27 +961,23 @@ void kick_sf(frost_ctx *c, Lane &M, Lane *Bl, const int32_t *S, int nS, const in
              bool gradient, double tau_pivot)
 {
     if (nS <= 0 || nF <= 0) return;
-    const bool tile = tile_force(c, nS, nF);
-    pack_acc(c, M, S, nS, M.recA, tile);
-    pack_acc(c, M, F, nF, M.recB, tile);
+    pack_acc(c, M, S, nS, M.recA);
+    pack_acc(c, M, F, nF, M.recB);
     Branch br(c, Bl ? Bl : &M, true);
     if (!Bl) br.concurrent = false;
     Lane &X = Bl ? br.exec : M;
     if (!gradient) {
         // each S x F pair once, when the symmetric grid fills the GPU
-        if (!tile && c->sym_cross >= 0 &&
-            pass_acc_sym(c, M, S, nS, F, nF, M.aA, M.aB, kick_of(c, S, cdt), kick_of(c, F, cdt), M.recA, M.recB,
-                         c->sym_cross > 0))
+        if (c->sym_cross >= 0 && pass_acc_sym(c, M, S, nS, F, nF, M.aA, M.aB, kick_of(c, S, cdt),
+                                              kick_of(c, F, cdt), M.recA, M.recB, c->sym_cross > 0))
             return;
         br.fork();
-        pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, nullptr, nullptr, kick_of(c, S, cdt), M.recA, M.recB, false,
-                 tile);
-        pass_acc(c, X, F, nF, S, nS, false, M.aB, nullptr, nullptr, nullptr, kick_of(c, F, cdt), M.recB, M.recA, false,
-                 tile);
+        pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, nullptr, nullptr, kick_of(c, S, cdt), M.recA, M.recB);
+        pass_acc(c, X, F, nF, S, nS, false, M.aB, nullptr, nullptr, nullptr, kick_of(c, F, cdt), M.recB, M.recA);
         return;  // joined by br
     }
     // each S x F pair once for both sides: always with sym_cross = 1, else for small lists
-    if (!tile && c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF <= kSymGradMaxPairs) &&
+    if (c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF <= kSymGradMaxPairs) &&
         grad_pairwise_sym(c, M, S, nS, F, nF, tau_pivot, M.atA, M.atB, nullptr, nullptr, nullptr, nullptr,
                           kick_of(c, S, cdt), kick_of(c, F, cdt), true))
         return;
@@ -1029,28 +985,28 @@ void kick_sf(frost_ctx *c, Lane &M, Lane *Bl, const int32_t *S, int nS, const in
     // the prepasses of both accurate passes in one symmetric kernel (each pair once), where
     // the lists are large
     bool wready = false;
-    if (!tile && c->mixed && c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF >= kSymCrossPrepassMinPairs)) {
+    if (c->mixed && c->sym_cross >= 0 && (c->sym_cross > 0 || (int64_t)nS * nF >= kSymCrossPrepassMinPairs)) {
         TimedScope ts(c, M.s, PASS_ACC, 0);
         launch_wmax_sym_cross(M.s, M.recA, nS, M.recB, nF, c->eps2, c->n_sm, M.wA, M.wB);
         c->st.kernel_launches += 1;
         wready = true;
     }
     br.fork();
-    pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, M.wA, h, KickArgs(), M.recA, M.recB, wready, tile);
+    pass_acc(c, M, S, nS, F, nF, false, M.aA, nullptr, M.wA, h, KickArgs(), M.recA, M.recB, wready);
     pass_acc(c, X, F, nF, S, nS, false, M.aB, nullptr, M.wB, h ? h + HOT_BINS : nullptr, KickArgs(), M.recB,
-             M.recA, wready, tile);
+             M.recA, wready);
     br.join();
     if (h) {
         mark_hot(c, M, nS, nF, false, M.aA, h, h + HOT_BINS, nF, M.hA);
         mark_hot(c, M, nF, nS, false, M.aB, h + HOT_BINS, h, nS, M.hB);
     }
-    pack_grad(c, M, S, nS, M.aA, M.recA, c->mixed ? M.hA : nullptr, tile);
-    pack_grad(c, M, F, nF, M.aB, M.recB, c->mixed ? M.hB : nullptr, tile);
+    pack_grad(c, M, S, nS, M.aA, M.recA, c->mixed ? M.hA : nullptr);
+    pack_grad(c, M, F, nF, M.aB, M.recB, c->mixed ? M.hB : nullptr);
     br.fork();
     pass_grad(c, M, S, nS, M.aA, F, nF, M.aB, false, tau_pivot, M.atA, nullptr, nullptr, M.wA, M.hB,
-              kick_of(c, S, cdt), M.recA, M.recB, tile);
+              kick_of(c, S, cdt), M.recA, M.recB);
     pass_grad(c, X, F, nF, M.aB, S, nS, M.aA, false, tau_pivot, M.atB, nullptr, nullptr, M.wB, M.hA,
-              kick_of(c, F, cdt), M.recB, M.recA, tile);
+              kick_of(c, F, cdt), M.recB, M.recA);
 }
 
 frost_status ensure_level(frost_ctx *c, int depth)
@@ -1611,8 +1567,6 @@ frost_status frost_accel_gradient(frost_ctx *c, const int32_t *active, int64_t n
         if (want_grad)
             pass_grad(c, M, P, nA, c->aA, P, nA, c->aA, true, eps_grad, nullptr, acc_tilde, grad, c->wA, c->hA,
                       KickArgs(), nullptr, nullptr, tile, omap);
-    } else if (want_grad && order_cross(c, nA, nB)) {
-        grad_pairwise_tile(c, M, A, nA, B, nB, eps_grad, acc, nullptr, acc_tilde, nullptr, grad, nullptr, true);
     } else if (want_grad && c->mixed && nB > 0 && c->sym_cross >= 0 &&
                (c->sym_cross > 0 || (int64_t)nA * nB >= kSymCrossPrepassMinPairs)) {
         // both accurate passes on records packed once, their prepasses in one symmetric kernel
@@ -1685,20 +1639,25 @@ frost_status frost_accel_gradient_pairwise(frost_ctx *c, const int32_t *a, int64
     if (c->hmisc->rel[0]) return fail(FROST_EINVAL, "index list has an out-of-range or repeated index");
     if (c->hmisc->rel[1] != 0) return fail(FROST_EINVAL, "the two lists share %lld particles", (long long)c->hmisc->rel[1]);
     Lane &M = c->main;
-    if (order_cross(c, nA, nB)) {
-        grad_pairwise_tile(c, M, A, nA, B, nB, eps_grad, acc_a, acc_b, acc_tilde_a, acc_tilde_b, grad_a, grad_b, false);
-    } else if (nA > 0 && nB > 0) {
+    if (nA > 0 && nB > 0) {
         pack_pos(c, M, A, nA, M.recA);
         pack_pos(c, M, B, nB, M.recB);
-        const bool sym = c->sym_cross >= 0 &&
+        const bool large = std::min(nA, nB) >= kOneSidedPairwiseMinN && (int64_t)nA * nB >= kOneSidedPairwiseMinPairs;
+        const bool sym = (c->sym_cross > 0 || (c->sym_cross == 0 && !large)) &&
                          grad_pairwise_sym(c, M, A, nA, B, nB, eps_grad, nullptr, nullptr, acc_tilde_a, acc_tilde_b,
                                            grad_a, grad_b, KickArgs(), KickArgs(), true);
         if (!sym) {
-            // two one-sided passes per kind, in the order of kick_sf
+            // two one-sided passes per kind, in the order of kick_sf (and with its prepass)
             unsigned *h = c->mixed ? zero_hists(M) : nullptr;
-            pass_acc(c, M, A, nA, B, nB, false, M.aA, nullptr, M.wA, h, KickArgs(), M.recA, M.recB);
+            const bool wready = c->mixed && c->sym_cross >= 0;
+            if (wready) {
+                TimedScope ts(c, M.s, PASS_ACC, 0);
+                launch_wmax_sym_cross(M.s, M.recA, nA, M.recB, nB, c->eps2, c->n_sm, M.wA, M.wB);
+                c->st.kernel_launches += 1;
+            }
+            pass_acc(c, M, A, nA, B, nB, false, M.aA, nullptr, M.wA, h, KickArgs(), M.recA, M.recB, wready);
             pass_acc(c, M, B, nB, A, nA, false, M.aB, nullptr, M.wB, h ? h + HOT_BINS : nullptr, KickArgs(), M.recB,
-                     M.recA);
+                     M.recA, wready);
             if (h) {
                 mark_hot(c, M, nA, nB, false, M.aA, h, h + HOT_BINS, nB, M.hA);
                 mark_hot(c, M, nB, nA, false, M.aB, h + HOT_BINS, h, nA, M.hB);
@@ -1796,7 +1755,7 @@ void leapfrog(frost_ctx *c, const int32_t *S, int nS, double h)
 {
     if (nS <= 0) return;
     Lane &M = c->main;
-    const bool tile = tile_force(c, nS, nS);
+    const bool tile = tile_force(c, nS);
     pass_acc(c, M, S, nS, S, nS, true, c->aA, nullptr, nullptr, nullptr, kick_of(c, S, 0.5 * h), nullptr, nullptr, false,
              tile);
     drift_pack(c, M, S, nS, h, c->recA, tile);

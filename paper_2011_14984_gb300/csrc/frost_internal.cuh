@@ -278,19 +278,18 @@ void launch_tstep_tile(cudaStream_t s, const int32_t *list, int n, const double 
                        int N, double G, double eta, int sym, int n_sm, void *rec, unsigned *best, const int32_t *pos,
                        double *tau, int *err);
 
-// Mixed Newtonian and gradient passes of spatially ordered lists (force_tiles.cu).  rec: tiles of
+// Mixed Newtonian and gradient passes of a spatially ordered list (force_tiles.cu).  rec: tiles of
 // TILE_N particles, TILE_POS_ROWS or TILE_GRAD_ROWS rows of TILE_N floats, then the tiles' heads.
 constexpr int TILE_N = 64;
 constexpr int TILE_POS_ROWS = 9, TILE_GRAD_ROWS = 13, TILE_HEAD_BYTES = 48;
 struct TileArgs {
-    const void *irec, *jrec;
-    int n_a, n_s;
-    int self_pass;   // 1 if the two lists are the same list
+    const void *rec;
+    int n;
     double eps2;     // softening^2
     int nsplit;      // j-splits (tile_splits)
-    double *part;    // partial results [nsplit][3][n_a]
+    double *part;    // partial results [nsplit][3][n]
 };
-int tile_splits(int n_a, int n_s, int n_sm, size_t part_elems);
+int tile_splits(int n, int n_sm, size_t part_elems);
 // position records; v (optional): after a drift by dt v (x is then written)
 void launch_tile_pack_pos(cudaStream_t s, const int32_t *list, int n, double *x, const double *v, double dt,
                           const double *m, int N, void *rec);

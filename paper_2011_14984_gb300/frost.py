@@ -392,7 +392,8 @@ class Frost:
     def accel_gradient_pairwise(self, a, b, eps_grad):
         """The force-gradient kick of the disjoint lists a and b due to each other: per list
         the Newtonian acceleration, a~ and the gradient ({"acc", "acc_tilde", "grad"} x
-        {"a", "b"}, [n][3] each); mixed mode: each pair once for both lists."""
+        {"a", "b"}, [n][3] each); mixed mode: each pair once for both lists (from 2^27 pairs of
+        two large lists on only with sym_cross = 1)."""
         t = self.torch
         A = self._dev(a, t.int32)
         B = self._dev(b, t.int32)

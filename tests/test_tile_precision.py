@@ -1,0 +1,29 @@
+"""GPU: what the tile passes of spatially ordered lists must not lose against the passes of every
+pair whose place they take: routes that the options promise, and precision."""
+import numpy as np
+import pytest
+
+from paper_2011_14984_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+
+
+def _frost(*args, **kw):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2011_14984_gb300.frost import Frost
+    return Frost(*args, **kw)
+
+
+def test_kicks_of_a_large_step_take_each_pair_once():
+    # the default of frost_opts.sym_cross: the two Newtonian kicks of the top level fill the GPU
+    n = 32768
+    m, x, v = ics.plummer(n, 3)
+    f = _frost(m, x, v)
+    tau = f.timesteps()
+    dt = float(tau.median())
+    slow, fast = f.partition(None, tau, dt)
+    f.reset_stats()
+    f.step(dt, 1)
+    assert f.stats()["acc_pairs_symmetric"] >= 2 * slow.numel() * fast.numel()
