@@ -101,14 +101,14 @@ typedef struct {
                                the mixed mode, the time-step pass of a set of at least 8192
                                particles evaluates each pair once for both particles (the same
                                result bits: the pair criteria are symmetric and a minimum does
-                               not depend on the order).  1: all always; -1: never.  (Mixed mode,
-                               contexts of at least 16384 particles: frost_step orders the
-                               particles in space before every top-level step, and the passes of
-                               large ordered lists, and of large lists given to the entry points,
-                               look at groups of particles through their boxes instead, in every
-                               mode of this option.  Time-steps keep their bits; forces keep the
-                               accuracy stated at frost_accel_gradient.  The exact fly-by
-                               derivative's time-steps stay as they are.) */
+                               not depend on the order).  In the mixed mode and contexts of at
+                               least 16384 particles, passes of one large list (from 8192
+                               particles in a step for time-steps and 4096 for forces, 16384 and
+                               24576 in the entry points) put it in spatial order instead and look
+                               at groups of particles through their boxes: time-steps keep their
+                               bits, forces the accuracy stated at frost_accel_gradient; the exact
+                               fly-by derivative's time-steps stay as they are.  1: each pair once
+                               in all these passes, at every size; -1: never, one-sided passes */
 } frost_opts;
 
 typedef enum {

@@ -443,8 +443,9 @@ void pack_pos(frost_ctx *c, Lane &L, const int32_t *list, int n, void *rec)
 
 int badbit(const frost_ctx *c) { return c->eps2 == 0.0 ? ERR_COINCIDENT : ERR_NONFINITE; }
 
-// whether an entry point puts a list of n particles in spatial order
-bool use_order(const frost_ctx *c, int n) { return c->ord && n >= kOrderMinN; }
+// whether a step or an entry point puts a list of n particles in spatial order, for the tile kernels;
+// frost_opts.sym_cross = 1 and -1 choose among the passes that look at every pair
+bool use_order(const frost_ctx *c, int n, int n_min = kOrderMinN) { return c->ord && c->sym_cross == 0 && n >= n_min; }
 
 void order_list(frost_ctx *c, const int32_t *list, int n, int32_t *pos, int32_t *sorted)
 {
@@ -1553,7 +1554,7 @@ frost_status frost_accel_gradient(frost_ctx *c, const int32_t *active, int64_t n
     Lane &M = c->main;
     if (self) {
         // a large set in spatial order, the results in the caller's
-        const bool tile = c->ord && nA >= kOrderForceMinN;
+        const bool tile = use_order(c, nA, kOrderForceMinN);
         const int32_t *P = A, *omap = nullptr;
         if (tile) {
             order_list(c, active, nA, c->opos, c->olist);
@@ -1984,7 +1985,7 @@ frost_status frost_energy_momentum(frost_ctx *c, double *E_kin, double *E_pot, d
         }
         return FROST_OK;
     }
-    if (use_order(c, c->N)) {
+    if (c->ord) {
         const int ns = potential_tile_splits(c->N, c->n_sm, c->part_elems);
         order_list(c, nullptr, c->N, c->opos, c->olist);
         launch_tile_pack_pos(c->stream, c->olist, c->N, c->x, nullptr, 0.0, c->m, c->N, c->recA);

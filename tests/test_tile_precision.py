@@ -27,3 +27,20 @@ def test_kicks_of_a_large_step_take_each_pair_once():
     f.reset_stats()
     f.step(dt, 1)
     assert f.stats()["acc_pairs_symmetric"] >= 2 * slow.numel() * fast.numel()
+
+
+@pytest.mark.parametrize("sym_cross", [1, -1])
+def test_sym_cross_chooses_the_passes_of_every_pair(sym_cross):
+    # always / never: the calls that would order a list launch what they launch one particle below
+    # the size from which they do (a sort alone would be four launches more)
+    def launches(n, call):
+        m, x, v = ics.plummer(n, 5)
+        f = _frost(m, x, v, sym_cross=sym_cross)
+        f.reset_stats()
+        call(f)
+        return f.stats()["kernel_launches"]
+
+    for n, call in ((16384, lambda f: f.timesteps()), (16384, lambda f: f.fsi(None, 2.0 ** -12)),
+                    (24576, lambda f: f.accel_gradient(eps_grad=0.05)),
+                    (24576, lambda f: f.accel_gradient(want=("acc",)))):
+        assert launches(n, call) == launches(n - 1, call)
