@@ -20,9 +20,8 @@
 //
 // Dominant terms (above 1/16 of max_j m_j / r^3, of the prepass) are kept out of the FP32 sums
 // and summed in double-float as in the other mixed passes.  In an ordered list they sit in the
-// few tiles around the receiver, so a receiver has more slots a split.  Only near tiles are
-// searched for them: a tile counts as far only if its heaviest mass at distance D stays below
-// every receiver's threshold.
+// few tiles around the receiver, so a receiver has more slots a split.  A tile is searched for
+// them unless its heaviest mass at its box stays below every receiver's threshold.
 // The prepass itself looks only at tiles whose box can hold a larger m_j / r^3.
 //
 // Pairs of sources are the two lanes of packed f32x2 instructions (tiles are structures of
@@ -41,6 +40,7 @@ constexpr int TJ = TILE_N;            // particles a tile: the 64 receivers of a
 static_assert(TJ == 64, "two particles a lane");
 constexpr int TB = TJ / 4;            // 16-byte pieces of a row
 constexpr float kFarRadius = 0.2f;    // far: box distance of at least this many source radii
+constexpr int SLOTS = 16;             // dominant terms a receiver and split (see Slots)
 constexpr float kFar = 1.0e15f;       // offset of the stand-ins past the end (mass 0)
 
 // rows of 64 floats of a tile: positions {x, y, z, m}, {low parts of x, y, z, m}, m^(-2/3)
@@ -286,6 +286,15 @@ __device__ __forceinline__ void four_roundings(float h, float l, float2 (&out)[2
     out[1] = make_float2(-a2, -a3);
 }
 
+// the negated receiver offset h + l for a searched tile: in a far one (single) its four roundings,
+// else both parts, which a near pair's separation needs
+__device__ __forceinline__ void searched_offset(bool single, float h, float l, float2 (&n)[2], float2 &nl)
+{
+    four_roundings(h, l, n);
+    if (!single) n[0] = n[1] = dup(-h);
+    nl = dup(single ? 0.f : -l);
+}
+
 __device__ __forceinline__ float2 half_of(const float4 v, int u) { return u ? make_float2(v.z, v.w) : make_float2(v.x, v.y); }
 
 // ------------------------------------------------------------------------------------
@@ -396,35 +405,56 @@ __global__ void __launch_bounds__(32) k_wmax_tile(const float *__restrict__ rec,
     }
 }
 
-// The next 32 tiles of a split: far (fm) and near (nm).  A tile is far from a receiver at
-// distance d >= kFarRadius R_J of its box and, with HEAVY, if it holds no dominant term to look
-// for: its heaviest mass at d stays below the receiver's threshold, d^2 m^(-2/3) > qk, or
-// d >= R_J, where its 64 terms are much alike (from outside a core, all of its terms are within
-// a factor 16 of the largest, and none of them dominates).  Box against box with the largest qk
-// (qthr) first, then, where that does not settle it, receiver by receiver.
+// The next 32 tiles of a split.  A tile is far from a receiver at distance d >= kFarRadius R_J of
+// its box.  fm: far from every receiver and, with HEAVY, without a dominant term to look for: its
+// heaviest mass at d stays below the receiver's threshold, d^2 m^(-2/3) > qk (qk = 0 for a
+// receiver without a free slot).  sm: the others, to be searched for dominant terms; lm: those
+// of sm that are far, which take single separations all the same.  Box against box with the
+// largest qk (qthr) first, then, where that does not settle it, receiver by receiver.
+// (Distance alone does not clear a tile: with a body of half the mass at the centre of a Plummer
+// sphere, tiles left unsearched from R_J on made the median error of a 17 times, of g 19 times
+// larger.)
 template <bool HEAVY>
 __device__ __forceinline__ void judge_tiles(const Group &W, const Head *__restrict__ jh, int ntiles, int t0, int nsplit,
                                             int own, bool live0, bool live1, float qthr, const float (&qk)[2], unsigned &fm,
-                                            unsigned &nm)
+                                            unsigned &sm, unsigned &lm)
 {
     const int t = t0 + (threadIdx.x & 31) * nsplit;
     bool far = false;
     if (t < ntiles && t != own) {
         const float4 c = jh[t].c, h = jh[t].h;
-        const float d2 = box_gap2(W.head.c, W.head.h, c, h), R2 = c.w * c.w;
-        far = d2 > 0.f && d2 >= (kFarRadius * kFarRadius) * R2 && (!HEAVY || d2 * h.w > qthr || d2 >= R2);
+        const float d2 = box_gap2(W.head.c, W.head.h, c, h);
+        far = d2 > 0.f && d2 >= (kFarRadius * kFarRadius) * (c.w * c.w) && (!HEAVY || d2 * h.w > qthr);
     }
     fm = __ballot_sync(kFull, far);
-    nm = 0u;
+    sm = lm = 0u;
     for (unsigned um = __ballot_sync(kFull, t < ntiles && !far); um; um &= um - 1) {
         const int b = __ffs(um) - 1, tt = t0 + b * nsplit;
         const float4 c = jh[tt].c, h = jh[tt].h;
-        const float R2 = c.w * c.w, d0 = point_gap2(W, 0, c, h), d1 = point_gap2(W, 1, c, h);
-        const bool ok0 = d0 > 0.f && d0 >= (kFarRadius * kFarRadius) * R2 && (!HEAVY || d0 * h.w > qk[0] || d0 >= R2);
-        const bool ok1 = d1 > 0.f && d1 >= (kFarRadius * kFarRadius) * R2 && (!HEAVY || d1 * h.w > qk[1] || d1 >= R2);
-        if (tt != own && __all_sync(kFull, (ok0 || !live0) && (ok1 || !live1))) fm |= 1u << b;
-        else nm |= 1u << b;
+        const float D2 = (kFarRadius * kFarRadius) * (c.w * c.w);
+        const float d0 = point_gap2(W, 0, c, h), d1 = point_gap2(W, 1, c, h);
+        const bool sep = ((d0 > 0.f && d0 >= D2) || !live0) && ((d1 > 0.f && d1 >= D2) || !live1);
+        const bool light = !HEAVY || ((d0 * h.w > qk[0] || !live0) && (d1 * h.w > qk[1] || !live1));
+        if (tt == own || !__all_sync(kFull, sep)) {
+            sm |= 1u << b;
+        } else if (HEAVY && !__all_sync(kFull, light)) {
+            sm |= 1u << b;
+            lm |= 1u << b;
+        } else {
+            fm |= 1u << b;
+        }
     }
+}
+
+// whether a receiver with a free slot may find a dominant term in the tile: a far tile is searched
+// only then (halo receivers, for which the whole core is within a factor 16 of the largest
+// term, fill their slots in a tile or two: acc+gradient of 65536 particles 8.13 -> 7.94 ms)
+__device__ __forceinline__ bool worth_search(const Group &W, const float4 c, const float4 h, bool live0, bool live1,
+                                             const float (&qk)[2], const int (&cnt)[2])
+{
+    const bool n0 = live0 && cnt[0] < SLOTS && !(point_gap2(W, 0, c, h) * h.w > qk[0]);
+    const bool n1 = live1 && cnt[1] < SLOTS && !(point_gap2(W, 1, c, h) * h.w > qk[1]);
+    return __any_sync(kFull, n0 || n1);
 }
 
 // ------------------------------------------------------------------------------------
@@ -435,7 +465,6 @@ __device__ __forceinline__ void judge_tiles(const Group &W, const Head *__restri
 // touched a few times per receiver and split.  The limit is for receivers far out in the halo,
 // for which thousands of sources are within a factor 16 of the nearest: their warps, without
 // it, made the 65536-body passes a third longer (32 slots: a step of 53.1 ms, 16: 52.3 ms).
-constexpr int SLOTS = 16;
 struct Slots {
     int j[2][SLOTS];
     float sum[2][6];
@@ -555,7 +584,8 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
     const int lane = threadIdx.x & 31, g = blockIdx.x, ntiles = (n + TJ - 1) / TJ;
     const Head *jh = heads(rec, n, P_ROWS);
     load_group(W, rec, n, P_ROWS, P_XL, g);
-    float thr[2] = {INFINITY, INFINITY}, qk[2] = {0.f, 0.f}, qthr = 0.f;
+    const bool live0 = g * TJ + slot_of(0) < n, live1 = g * TJ + slot_of(1) < n;
+    float thr[2] = {INFINITY, INFINITY}, qk[2] = {0.f, 0.f};
     int cnt[2] = {0, 0};
     if (ACC) {
 #pragma unroll
@@ -564,16 +594,15 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
         // r^2 m^(-2/3) at the threshold: a pair above it is below the threshold
 #pragma unroll
         for (int k = 0; k < 2; ++k) qk[k] = 1.0001f * exp2f(-0.6666667f * log2f(thr[k]));
-        qthr = warp_max(fmaxf(qk[0], qk[1]));
         slots_clear(S);
     }
     const float2 e2 = dup(eps2);
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
-        unsigned fm, nm;
-        judge_tiles<ACC>(W, jh, ntiles, t0, nsplit, g, g * TJ + slot_of(0) < n, g * TJ + slot_of(1) < n, qthr,
-                         qk, fm, nm);
+        unsigned fm, sm, lm;
+        const float qf[2] = {cnt[0] < SLOTS ? qk[0] : 0.f, cnt[1] < SLOTS ? qk[1] : 0.f};
+        judge_tiles<ACC>(W, jh, ntiles, t0, nsplit, g, live0, live1, ACC ? warp_max(fmaxf(qf[0], qf[1])) : 0.f, qf, fm, sm, lm);
         // the next tile's rows wait in registers: 64 pieces of the far rows, 128 of all
-        auto next_bit = [&]() { return fm ? __ffs(fm) - 1 : __ffs(nm) - 1; };
+        auto next_bit = [&]() { return __ffs(fm ? fm : sm) - 1; };
         float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
         auto fetch = [&]() {
             const float4 *tr = (const float4 *)(rec + (size_t)(t0 + next_bit() * nsplit) * P_ROWS * TJ);
@@ -584,12 +613,13 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                 n3 = tr[96 + lane];
             }
         };
-        if (fm | nm) fetch();
-        while (fm | nm) {
+        if (fm | sm) fetch();
+        while (fm | sm) {
             const bool isfar = fm != 0u;
+            const bool single = (lm >> next_bit()) & 1u;
             const int t = t0 + next_bit() * nsplit;
             if (fm) fm &= fm - 1;
-            else nm &= nm - 1;
+            else sm &= sm - 1;
             const float4 c = jh[t].c;
             float4 *sf = &s[0][0];
             __syncwarp();
@@ -600,7 +630,7 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                 sf[96 + lane] = n3;
             }
             __syncwarp();
-            if (fm | nm) fetch();
+            if (fm | sm) fetch();
             float xh[2][3], xl[2][3];
             offsets(W, c, xh, xl);
             // ACC: four partial sums a component and tile (two accumulators of two lanes)
@@ -610,7 +640,7 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
             for (int k = 0; k < 2; ++k)
 #pragma unroll
                 for (int u = 0; u < NU; ++u) ax[k][u] = ay[k][u] = az[k][u] = dup(0.f);
-            if (isfar) {
+            if (isfar || (ACC && single && !worth_search(W, c, jh[t].h, live0, live1, qk, cnt))) {
                 float2 nx[2][3][2];
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
@@ -640,6 +670,11 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                 }
             } else {
                 const bool diag = t == g;
+                float2 nx[2][3][2], nl[2][3];
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) searched_offset(single, xh[k][q], xl[k][q], nx[k][q], nl[k][q]);
 #pragma unroll 1
                 for (int b = 0; b < TB; ++b) {
                     const float4 X = s[P_X][b], Y = s[P_Y][b], Z = s[P_Z][b], M = s[P_M][b];
@@ -648,12 +683,12 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                     for (int k = 0; k < 2; ++k)
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
-                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), dup(-xh[k][0])),
-                                                         __fadd2_rn(half_of(XL, u), dup(-xl[k][0])));
-                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), dup(-xh[k][1])),
-                                                         __fadd2_rn(half_of(YL, u), dup(-xl[k][1])));
-                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), dup(-xh[k][2])),
-                                                         __fadd2_rn(half_of(ZL, u), dup(-xl[k][2])));
+                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0][u]),
+                                                         __fadd2_rn(half_of(XL, u), nl[k][0]));
+                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1][u]),
+                                                         __fadd2_rn(half_of(YL, u), nl[k][1]));
+                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2][u]),
+                                                         __fadd2_rn(half_of(ZL, u), nl[k][2]));
                             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
                             float2 w = pair_weight<ACC>(r2, half_of(M, u));
                             const int j = t * TJ + 4 * b + 2 * u;
@@ -781,6 +816,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
             A.h[q][slot_of(k)] = rec[((size_t)g * G_ROWS + G_AX + q) * TJ + slot_of(k)];
             A.l[q][slot_of(k)] = rec[((size_t)g * G_ROWS + G_AXL + q) * TJ + slot_of(k)];
         }
+    const bool live0 = g * TJ + slot_of(0) < n, live1 = g * TJ + slot_of(1) < n;
     float thr[2] = {INFINITY, INFINITY};
     int cnt[2] = {0, 0};
 #pragma unroll
@@ -789,14 +825,13 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
     float qk[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) qk[k] = 1.0001f * exp2f(-0.6666667f * log2f(thr[k]));
-    const float qthr = warp_max(fmaxf(qk[0], qk[1]));
     slots_clear(S);
     const float2 e2 = dup((float)eps2d);
     for (int t0 = blockIdx.y; t0 < ntiles; t0 += 32 * nsplit) {
-        unsigned fm, nm;
-        judge_tiles<true>(W, jh, ntiles, t0, nsplit, g, g * TJ + slot_of(0) < n, g * TJ + slot_of(1) < n, qthr,
-                         qk, fm, nm);
-        auto next_bit = [&]() { return fm ? __ffs(fm) - 1 : __ffs(nm) - 1; };
+        unsigned fm, sm, lm;
+        const float qf[2] = {cnt[0] < SLOTS ? qk[0] : 0.f, cnt[1] < SLOTS ? qk[1] : 0.f};
+        judge_tiles<true>(W, jh, ntiles, t0, nsplit, g, live0, live1, warp_max(fmaxf(qf[0], qf[1])), qf, fm, sm, lm);
+        auto next_bit = [&]() { return __ffs(fm ? fm : sm) - 1; };
         // the next tile's far rows wait in registers, 112 of its 208 pieces
         float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0, n2 = n0, n3 = n0;
         auto fetch = [&]() {
@@ -806,12 +841,13 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
             n2 = tr[64 + lane];
             n3 = tr[96 + lane];
         };
-        if (fm | nm) fetch();
-        while (fm | nm) {
+        if (fm | sm) fetch();
+        while (fm | sm) {
             const bool isfar = fm != 0u;
+            const bool single = (lm >> next_bit()) & 1u;
             const int t = t0 + next_bit() * nsplit;
             if (fm) fm &= fm - 1;
-            else nm &= nm - 1;
+            else sm &= sm - 1;
             const float4 c = jh[t].c, a = jh[t].a;
             float4 *sf = &s[0][0];
             __syncwarp();
@@ -826,7 +862,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                 if (lane < 16) sf[192 + lane] = tr[192 + lane];
             }
             __syncwarp();
-            if (fm | nm) fetch();
+            if (fm | sm) fetch();
             float xh[2][3], xl[2][3];
             offsets(W, c, xh, xl);
             // the receivers' accelerations less the tile's mean
@@ -851,7 +887,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
             for (int k = 0; k < 2; ++k)
 #pragma unroll
                 for (int u = 0; u < 2; ++u) gx[k][u] = gy[k][u] = gz[k][u] = dup(0.f);
-            if (isfar) {
+            if (isfar || (single && !worth_search(W, c, jh[t].h, live0, live1, qk, cnt))) {
                 float2 nx[2][3][2], na[2][3][2];
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
@@ -886,6 +922,14 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                 }
             } else {
                 const bool diag = t == g;
+                float2 nx[2][3][2], nl[2][3], na[2][3][2], ma[2][3];
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        searched_offset(single, xh[k][q], xl[k][q], nx[k][q], nl[k][q]);
+                        searched_offset(single, Ah[k][q], Al[k][q], na[k][q], ma[k][q]);
+                    }
 #pragma unroll 1
                 for (int b = 0; b < TB; ++b) {
                     const float4 X = s[G_X][b], Y = s[G_Y][b], Z = s[G_Z][b], M = s[G_M][b];
@@ -897,12 +941,12 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
 #define half_of(V, u) (half_of(V, u))
-                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), dup(-xh[k][0])), __fadd2_rn(half_of(XL, u), dup(-xl[k][0])));
-                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), dup(-xh[k][1])), __fadd2_rn(half_of(YL, u), dup(-xl[k][1])));
-                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), dup(-xh[k][2])), __fadd2_rn(half_of(ZL, u), dup(-xl[k][2])));
-                            const float2 Ax = __fadd2_rn(__fadd2_rn(half_of(P, u), dup(-Ah[k][0])), __fadd2_rn(half_of(PL, u), dup(-Al[k][0])));
-                            const float2 Ay = __fadd2_rn(__fadd2_rn(half_of(Q, u), dup(-Ah[k][1])), __fadd2_rn(half_of(QL, u), dup(-Al[k][1])));
-                            const float2 Az = __fadd2_rn(__fadd2_rn(half_of(R, u), dup(-Ah[k][2])), __fadd2_rn(half_of(RL, u), dup(-Al[k][2])));
+                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0][u]), __fadd2_rn(half_of(XL, u), nl[k][0]));
+                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1][u]), __fadd2_rn(half_of(YL, u), nl[k][1]));
+                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2][u]), __fadd2_rn(half_of(ZL, u), nl[k][2]));
+                            const float2 Ax = __fadd2_rn(__fadd2_rn(half_of(P, u), na[k][0][u]), __fadd2_rn(half_of(PL, u), ma[k][0]));
+                            const float2 Ay = __fadd2_rn(__fadd2_rn(half_of(Q, u), na[k][1][u]), __fadd2_rn(half_of(QL, u), ma[k][1]));
+                            const float2 Az = __fadd2_rn(__fadd2_rn(half_of(R, u), na[k][2][u]), __fadd2_rn(half_of(RL, u), ma[k][2]));
                             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
                             float2 w, ri2;
                             grad_weight(r2, half_of(M, u), w, ri2);

@@ -44,3 +44,20 @@ def test_sym_cross_chooses_the_passes_of_every_pair(sym_cross):
                     (24576, lambda f: f.accel_gradient(eps_grad=0.05)),
                     (24576, lambda f: f.accel_gradient(want=("acc",)))):
         assert launches(n, call) == launches(n - 1, call)
+
+
+@pytest.mark.parametrize("n", [24577, 32768])
+def test_a_dominant_mass_stays_in_double_float(n):
+    # half of the mass in one body: its term is most of nearly every particle's a and g.  Any one FP32
+    # evaluation of that term would leave a relative error of about 2^-24 (half a unit each of
+    # separation, r^2, its root and the product); summed in double-float, what is left are the FP32
+    # terms of the others, thousands of which share the rest.  A quarter of 2^-24 lies between.
+    m, x, v = ics.plummer(n, 31, ics.kroupa_masses(n, 31))
+    m = 0.5 * m / m[1:].sum()
+    m[0] = 0.5
+    x[0] *= 0.01
+    out = _frost(m, x, v).accel_gradient(eps_grad=0.05)
+    ref = _frost(m, x, v, precision="fp64").accel_gradient(eps_grad=0.05)
+    for key in ("acc", "grad"):
+        o, r = out[key].cpu().numpy()[1:], ref[key].cpu().numpy()[1:]
+        assert np.median(np.linalg.norm(o - r, axis=1) / np.linalg.norm(r, axis=1)) < 2.0 ** -26, key
