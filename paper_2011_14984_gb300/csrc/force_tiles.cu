@@ -8,15 +8,17 @@
 // 2^-24 of a distance that may be far smaller.  Here a tile's positions are kept relative to its
 // own centre c_J (hi + lo, 48 bits of an offset of at most the tile's radius R_J), and a
 // receiver's offset X = x_i - c_J is formed once a tile, in double-float, for 64 pairs:
-//   far tile (box distance D >= R_J / 5): dx = x'_j - X with both rounded to FP32, one addition.
-//     The rounding of x'_j is below 2^-25 R_J, that of X below 2^-25 (|dx| + R_J).
+//   far tile (box distance D >= R_J / 5): dx = (x'_j - X_lo) - X_hi, x'_j rounded to FP32: two
+//     additions, and below 2^-25 (|dx| + 2 R_J) in error.  (The low part first: added last, or to
+//     a high difference that is already on the grid of dx, it is lost, the same way for every
+//     source of the tile, and such errors add up.  One addition of a rounding of X, four
+//     roundings in turn whose mean is right, scatter so much that g was off by 1.13 times the
+//     one-sided pass's error at the 99.9th percentile; now 0.78.)
 //   near tile: dx = (x'_j,hi - X_hi) + (x'_j,lo - X_lo), three additions as before.
-// The gradient's a_j - a_i works alike against a tile's mean acceleration: one addition instead
-// of three in far tiles.  A rounding of X or of the receiver's acceleration is the same for all
-// pairs of a tile, and such errors add up where a far particle's sum over the tiles cancels; so
-// the four sources of a step of a far tile's loop take four roundings of each whose mean is
-// right to an eighth of a unit.  For the same reason a tile's terms, which all point the same
-// way, are summed in four partial sums of 16, two of which share a compensated sum.
+// The gradient's a_j - a_i works alike against a tile's mean acceleration.  The plain Newtonian
+// pass, whose error is the MUFU rsqrt's, does take the four roundings of X.
+// A tile's terms, which all point the same way, are summed in four partial sums of 16, two of
+// which share a compensated sum.
 //
 // Dominant terms (above 1/16 of max_j m_j / r^3, of the prepass) are kept out of the FP32 sums
 // and summed in double-float as in the other mixed passes.  In an ordered list they sit in the
@@ -286,13 +288,20 @@ __device__ __forceinline__ void four_roundings(float h, float l, float2 (&out)[2
     out[1] = make_float2(-a2, -a3);
 }
 
-// the negated receiver offset h + l for a searched tile: in a far one (single) its four roundings,
-// else both parts, which a near pair's separation needs
-__device__ __forceinline__ void searched_offset(bool single, float h, float l, float2 (&n)[2], float2 &nl)
+// a separation in a far tile: x'_j less the receiver's low part, then less its high part (LOW),
+// or x'_j less one of four roundings
+template <bool LOW>
+__device__ __forceinline__ float2 far_sep(float2 x, const float2 (&n)[2], int u)
 {
-    four_roundings(h, l, n);
-    if (!single) n[0] = n[1] = dup(-h);
-    nl = dup(single ? 0.f : -l);
+    return LOW ? __fadd2_rn(__fadd2_rn(x, n[1]), n[0]) : __fadd2_rn(x, n[u]);
+}
+
+// the negated receiver offset h + l for a searched tile, the part that goes with the sources' high
+// parts first: in a far tile (single) the low one
+__device__ __forceinline__ void searched_offset(bool single, float h, float l, float2 &nh, float2 &nl)
+{
+    nh = dup(single ? -l : -h);
+    nl = dup(single ? -h : -l);
 }
 
 __device__ __forceinline__ float2 half_of(const float4 v, int u) { return u ? make_float2(v.z, v.w) : make_float2(v.x, v.y); }
@@ -641,15 +650,20 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
 #pragma unroll
                 for (int u = 0; u < NU; ++u) ax[k][u] = ay[k][u] = az[k][u] = dup(0.f);
             if (isfar || (ACC && single && !worth_search(W, c, jh[t].h, live0, live1, qk, cnt))) {
+                // ACC: {-high part, -low part}; else four roundings (an addition a component less,
+                // with an error of a below that of the MUFU rsqrt; one rounding for all
+                // sources had a median error 2 % above the one-sided pass's, four 5 % below it)
                 float2 nx[2][3][2];
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        // the plain pass keeps one rounding (4 % faster, and within the error of
-                        // the MUFU rsqrt)
-                        if (ACC) four_roundings(xh[k][q], xl[k][q], nx[k][q]);
-                        else nx[k][q][0] = nx[k][q][1] = dup(-__fadd_rn(xh[k][q], xl[k][q]));
+                        if (ACC) {
+                            nx[k][q][0] = dup(-xh[k][q]);
+                            nx[k][q][1] = dup(-xl[k][q]);
+                        } else {
+                            four_roundings(xh[k][q], xl[k][q], nx[k][q]);
+                        }
                     }
 #pragma unroll 2
                 for (int b = 0; b < TB; ++b) {
@@ -658,9 +672,9 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                     for (int k = 0; k < 2; ++k)
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
-                            const float2 dx = __fadd2_rn(half_of(X, u), nx[k][0][u]);
-                            const float2 dy = __fadd2_rn(half_of(Y, u), nx[k][1][u]);
-                            const float2 dz = __fadd2_rn(half_of(Z, u), nx[k][2][u]);
+                            const float2 dx = far_sep<ACC>(half_of(X, u), nx[k][0], u);
+                            const float2 dy = far_sep<ACC>(half_of(Y, u), nx[k][1], u);
+                            const float2 dz = far_sep<ACC>(half_of(Z, u), nx[k][2], u);
                             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
                             const float2 w = pair_weight<ACC>(r2, half_of(M, u));
                             ax[k][u % NU] = __ffma2_rn(w, dx, ax[k][u % NU]);
@@ -670,7 +684,7 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                 }
             } else {
                 const bool diag = t == g;
-                float2 nx[2][3][2], nl[2][3];
+                float2 nx[2][3], nl[2][3];
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
@@ -683,11 +697,11 @@ __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__r
                     for (int k = 0; k < 2; ++k)
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
-                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0][u]),
+                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0]),
                                                          __fadd2_rn(half_of(XL, u), nl[k][0]));
-                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1][u]),
+                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1]),
                                                          __fadd2_rn(half_of(YL, u), nl[k][1]));
-                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2][u]),
+                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2]),
                                                          __fadd2_rn(half_of(ZL, u), nl[k][2]));
                             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
                             float2 w = pair_weight<ACC>(r2, half_of(M, u));
@@ -893,8 +907,10 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        four_roundings(xh[k][q], xl[k][q], nx[k][q]);
-                        four_roundings(Ah[k][q], Al[k][q], na[k][q]);
+                        nx[k][q][0] = dup(-xh[k][q]);
+                        nx[k][q][1] = dup(-xl[k][q]);
+                        na[k][q][0] = dup(-Ah[k][q]);
+                        na[k][q][1] = dup(-Al[k][q]);
                     }
 #pragma unroll 2
                 for (int b = 0; b < TB; ++b) {
@@ -904,12 +920,12 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                     for (int k = 0; k < 2; ++k)
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
-                            const float2 dx = __fadd2_rn(half_of(X, u), nx[k][0][u]);
-                            const float2 dy = __fadd2_rn(half_of(Y, u), nx[k][1][u]);
-                            const float2 dz = __fadd2_rn(half_of(Z, u), nx[k][2][u]);
-                            const float2 Ax = __fadd2_rn(half_of(P, u), na[k][0][u]);
-                            const float2 Ay = __fadd2_rn(half_of(Q, u), na[k][1][u]);
-                            const float2 Az = __fadd2_rn(half_of(R, u), na[k][2][u]);
+                            const float2 dx = far_sep<true>(half_of(X, u), nx[k][0], u);
+                            const float2 dy = far_sep<true>(half_of(Y, u), nx[k][1], u);
+                            const float2 dz = far_sep<true>(half_of(Z, u), nx[k][2], u);
+                            const float2 Ax = far_sep<true>(half_of(P, u), na[k][0], u);
+                            const float2 Ay = far_sep<true>(half_of(Q, u), na[k][1], u);
+                            const float2 Az = far_sep<true>(half_of(R, u), na[k][2], u);
                             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
                             float2 w, ri2;
                             grad_weight(r2, half_of(M, u), w, ri2);
@@ -922,7 +938,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                 }
             } else {
                 const bool diag = t == g;
-                float2 nx[2][3][2], nl[2][3], na[2][3][2], ma[2][3];
+                float2 nx[2][3], nl[2][3], na[2][3], ma[2][3];
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
@@ -941,12 +957,12 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
 #define half_of(V, u) (half_of(V, u))
-                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0][u]), __fadd2_rn(half_of(XL, u), nl[k][0]));
-                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1][u]), __fadd2_rn(half_of(YL, u), nl[k][1]));
-                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2][u]), __fadd2_rn(half_of(ZL, u), nl[k][2]));
-                            const float2 Ax = __fadd2_rn(__fadd2_rn(half_of(P, u), na[k][0][u]), __fadd2_rn(half_of(PL, u), ma[k][0]));
-                            const float2 Ay = __fadd2_rn(__fadd2_rn(half_of(Q, u), na[k][1][u]), __fadd2_rn(half_of(QL, u), ma[k][1]));
-                            const float2 Az = __fadd2_rn(__fadd2_rn(half_of(R, u), na[k][2][u]), __fadd2_rn(half_of(RL, u), ma[k][2]));
+                            const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0]), __fadd2_rn(half_of(XL, u), nl[k][0]));
+                            const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1]), __fadd2_rn(half_of(YL, u), nl[k][1]));
+                            const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2]), __fadd2_rn(half_of(ZL, u), nl[k][2]));
+                            const float2 Ax = __fadd2_rn(__fadd2_rn(half_of(P, u), na[k][0]), __fadd2_rn(half_of(PL, u), ma[k][0]));
+                            const float2 Ay = __fadd2_rn(__fadd2_rn(half_of(Q, u), na[k][1]), __fadd2_rn(half_of(QL, u), ma[k][1]));
+                            const float2 Az = __fadd2_rn(__fadd2_rn(half_of(R, u), na[k][2]), __fadd2_rn(half_of(RL, u), ma[k][2]));
                             const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
                             float2 w, ri2;
                             grad_weight(r2, half_of(M, u), w, ri2);

@@ -61,3 +61,24 @@ def test_a_dominant_mass_stays_in_double_float(n):
     for key in ("acc", "grad"):
         o, r = out[key].cpu().numpy()[1:], ref[key].cpu().numpy()[1:]
         assert np.median(np.linalg.norm(o - r, axis=1) / np.linalg.norm(r, axis=1)) < 2.0 ** -26, key
+
+
+def _errors(f, ref, want):
+    out = f.accel_gradient(eps_grad=0.05) if want != "plain" else {"plain": f.accel_gradient(want=("acc",))["acc"]}
+    o, r = out[want].cpu().numpy(), ref["acc" if want == "plain" else want].cpu().numpy()
+    return np.linalg.norm(o - r, axis=1) / np.linalg.norm(r, axis=1)
+
+
+# what the one-sided passes of every pair (sym_cross = -1) reach is the bar: over the particles of
+# three systems together, no quantile of the error may be larger
+@pytest.mark.parametrize("masses,want", [("equal", "grad"), ("kroupa", "grad"), ("kroupa", "plain")])
+def test_tile_passes_are_as_precise_as_the_passes_of_every_pair(masses, want):
+    n = 65536
+    err = {0: [], -1: []}
+    for seed in (41, 42, 43):
+        m, x, v = ics.plummer(n, seed, ics.kroupa_masses(n, seed) if masses == "kroupa" else None)
+        ref = _frost(m, x, v, precision="fp64").accel_gradient(eps_grad=0.05)
+        for sc in err:
+            err[sc].append(_errors(_frost(m, x, v, sym_cross=sc), ref, want))
+    for q in (0.5, 0.99, 0.999):
+        assert np.quantile(np.concatenate(err[0]), q) <= np.quantile(np.concatenate(err[-1]), q), q
