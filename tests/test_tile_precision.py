@@ -71,7 +71,8 @@ def _errors(f, ref, want):
 
 # what the one-sided passes of every pair (sym_cross = -1) reach is the bar: over the particles of
 # three systems together, no quantile of the error may be larger
-@pytest.mark.parametrize("masses,want", [("equal", "grad"), ("kroupa", "grad"), ("kroupa", "plain")])
+@pytest.mark.parametrize("masses,want", [("equal", "grad"), ("kroupa", "grad"), ("kroupa", "plain"),
+                                         ("kroupa", "acc"), ("equal", "acc")])
 def test_tile_passes_are_as_precise_as_the_passes_of_every_pair(masses, want):
     n = 65536
     err = {0: [], -1: []}
