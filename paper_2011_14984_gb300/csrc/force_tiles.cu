@@ -32,6 +32,7 @@
 // What a tile costs beside its pairs (offsets, roundings, folds: about 250 instructions) is why it
 // holds 64 sources: with 32 it was 45 % of the instructions executed.
 #include "pair_bodies.cuh"
+#include "tile_bounds.cuh"
 
 namespace frost {
 namespace {
@@ -80,16 +81,10 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
-// The squared distance of two boxes, from below: centres and half sizes are FP32 values, so the
-// gap is good to a few units whatever the distance of the tiles from the origin
-__device__ __forceinline__ float axis_gap(float d, float h) { return fmaxf(0.f, fmaf(fabsf(d), 0.999999f, -1.000001f * h)); }
-
+// the squared distance of two boxes, from below
 __device__ __forceinline__ float box_gap2(const float4 ca, const float4 ha, const float4 cb, const float4 hb)
 {
-    const float gx = axis_gap(ca.x - cb.x, ha.x + hb.x);
-    const float gy = axis_gap(ca.y - cb.y, ha.y + hb.y);
-    const float gz = axis_gap(ca.z - cb.z, ha.z + hb.z);
-    return fmaf(gx, gx, fmaf(gy, gy, gz * gz));
+    return gap2(axis_gap(ca.x - cb.x, ha.x + hb.x), axis_gap(ca.y - cb.y, ha.y + hb.y), axis_gap(ca.z - cb.z, ha.z + hb.z));
 }
 
 // ------------------------------------------------------------------------------------
@@ -268,10 +263,8 @@ __device__ __forceinline__ double group_total(const Group &W, int q, int r)
 __device__ __forceinline__ float point_gap2(const Group &W, int k, const float4 c, const float4 h)
 {
     const int r = slot_of(k);
-    const float gx = axis_gap((W.head.c.x - c.x) + W.xh[0][r], h.x);
-    const float gy = axis_gap((W.head.c.y - c.y) + W.xh[1][r], h.y);
-    const float gz = axis_gap((W.head.c.z - c.z) + W.xh[2][r], h.z);
-    return fmaf(gx, gx, fmaf(gy, gy, gz * gz));
+    return gap2(point_axis_gap(W.head.c.x - c.x, W.xh[0][r], h.x), point_axis_gap(W.head.c.y - c.y, W.xh[1][r], h.y),
+                point_axis_gap(W.head.c.z - c.z, W.xh[2][r], h.z));
 }
 
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
