@@ -982,7 +982,6 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
                     for (int k = 0; k < 2; ++k)
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
-#define half_of(V, u) (half_of(V, u))
                             const float2 dx = __fadd2_rn(__fadd2_rn(half_of(X, u), nx[k][0]), __fadd2_rn(half_of(XL, u), nl[k][0]));
                             const float2 dy = __fadd2_rn(__fadd2_rn(half_of(Y, u), nx[k][1]), __fadd2_rn(half_of(YL, u), nl[k][1]));
                             const float2 dz = __fadd2_rn(__fadd2_rn(half_of(Z, u), nx[k][2]), __fadd2_rn(half_of(ZL, u), nl[k][2]));
