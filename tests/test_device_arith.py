@@ -12,9 +12,10 @@ CSRC = os.path.join(ROOT, "paper_2011_14984_gb300", "csrc")
 
 def _host_library(tmp_path, source):
     src, lib = tmp_path / "host.cc", tmp_path / "host.so"
+    (tmp_path / "cuda_runtime.h").write_text("")
     src.write_text("#define __host__\n#define __device__\n#define __forceinline__ inline\n" + source)
-    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-shared", "-fPIC", f"-I{CSRC}", str(src),
-                    "-o", str(lib)], check=True)
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-shared", "-fPIC", f"-I{tmp_path}", f"-I{CSRC}",
+                    str(src), "-o", str(lib)], check=True)
     return ctypes.CDLL(str(lib))
 
 
@@ -55,3 +56,53 @@ extern "C" void gaps(int n, const float *dc, const float *x, const float *h, flo
     margin = 2e-6 * (np.abs(dc) + np.abs(x) + h)
     least = np.maximum(0.0, exact - margin)
     assert np.all(out >= (least ** 2).sum(axis=1) * (1 - 1e-6))
+
+
+def test_integer_conversions_are_the_casts(tmp_path):
+    # the bits of (double)f and (float)d: FP32 values over all exponents and signs, FP64 values around
+    # every exponent of the FP32 range with the fractions that decide a rounding (ties to even both
+    # ways, one unit to either side, carries into the next exponent), zeros, the normal range's ends
+    lib = _host_library(tmp_path, """
+#include <cmath>
+#include <cstdint>
+#include <cstring>
+static unsigned __float_as_uint(float f) { unsigned u; std::memcpy(&u, &f, 4); return u; }
+static float __uint_as_float(unsigned u) { float f; std::memcpy(&f, &u, 4); return f; }
+static double __hiloint2double(int hi, int lo)
+{
+    const uint64_t u = ((uint64_t)(unsigned)hi << 32) | (unsigned)lo;
+    double d; std::memcpy(&d, &u, 8); return d;
+}
+static int __double2hiint(double d) { uint64_t u; std::memcpy(&u, &d, 8); return (int)(u >> 32); }
+static int __double2loint(double d) { uint64_t u; std::memcpy(&u, &d, 8); return (int)u; }
+static float __fadd_rn(float a, float b) { return a + b; }
+static float __fsub_rn(float a, float b) { return a - b; }
+static float __fmul_rn(float a, float b) { return a * b; }
+static float rsqrtf(float a) { return 1.f / std::sqrt(a); }
+#include "df_arith.cuh"
+extern "C" void to_double(int n, const float *f, double *d) { for (int i = 0; i < n; ++i) d[i] = frost::df::f2d(f[i]); }
+extern "C" void to_float(int n, const double *d, float *f) { for (int i = 0; i < n; ++i) f[i] = frost::df::d2f(d[i]); }
+""")
+    rng = np.random.default_rng(9)
+    expo = np.arange(256, dtype=np.uint32)
+    frac = np.concatenate([[0, 1, 2, 0x3fffff, 0x400000, 0x7ffffe, 0x7fffff],
+                           rng.integers(0, 1 << 23, 249)]).astype(np.uint32)
+    bits = ((expo[:, None] << 23) | frac[None, :]).ravel()
+    bits = np.concatenate([bits, bits | np.uint32(0x80000000)])
+    f = np.ascontiguousarray(bits).view(np.float32)
+    d = np.empty(f.size)
+    lib.to_double(f.size, _p(f), _p(d))
+    assert np.array_equal(d, f.astype(np.float64), equal_nan=True) and np.array_equal(np.signbit(d), np.signbit(f))
+
+    expo = np.concatenate([np.arange(880, 1170), [0, 1, 2046, 2047]]).astype(np.uint64)
+    high = np.concatenate([[0, 1, 2, (1 << 23) - 2, (1 << 23) - 1], rng.integers(0, 1 << 23, 59)]).astype(np.uint64)
+    low = np.concatenate([[0, 1, (1 << 28) - 1, 1 << 28, (1 << 28) + 1, (1 << 29) - 1],
+                          rng.integers(0, 1 << 29, 26)]).astype(np.uint64)
+    bits = ((expo[:, None, None] << np.uint64(52)) | (high[None, :, None] << np.uint64(29)) | low[None, None, :]).ravel()
+    bits = np.concatenate([bits, bits | np.uint64(1 << 63)])
+    d = np.ascontiguousarray(bits).view(np.float64)
+    f = np.empty(d.size, np.float32)
+    lib.to_float(d.size, _p(d), _p(f))
+    with np.errstate(over="ignore", invalid="ignore"):
+        r = d.astype(np.float32)
+    assert np.array_equal(f, r, equal_nan=True) and np.array_equal(np.signbit(f), np.signbit(r))
