@@ -41,9 +41,9 @@ FP64_PEAK_TFLOPS = 1.25  # nominal GB300 FP64 rate
 METRIC = "acc+gradient interactions/s"
 UNIT = "interactions/s"
 # DRAM bytes (read + write) per launch of the Newtonian kind in one 64k hierarchical step:
-# ncu dram__bytes_read.sum + dram__bytes_write.sum over the step's 396 launches of that kind,
-# captured on the current kernels
-TRAFFIC_ACC_PLUMMER64K = 388752.0
+# ncu dram__bytes_read.sum + dram__bytes_write.sum over the step's 396 launches of that kind (tiles,
+# symmetric and one-sided passes and the prepasses)
+TRAFFIC_ACC_PLUMMER64K = 407376.0
 
 
 # the bars the GPU tests hold the CUDA path to against the FP64 oracle (tests/test_gpu_parity.py)
@@ -520,7 +520,8 @@ def run_frost(args):
                            "subtree_max": args.subtree_max or "library default",
                            "integrator": args.integrator,
                            "branch_streams": "concurrent" if args.branch_streams >= 0 else "one stream",
-                           "sym_cross": {0: "where it fills the GPU", 1: "always", -1: "off"}[max(-1, min(1, args.sym_cross))],
+                           "sym_cross": {0: "where it fills the GPU; passes of one large list by tiles", 1: "always",
+                                         -1: "off"}[max(-1, min(1, args.sym_cross))],
                            "flyby_derivative": "exact" if args.flyby_exact else "two-body"},
                 "roofline": roofline, "cpu_baseline": cpu,
                 "e2e": {"value": e2e_value, "unit": UNIT, "steps": e2e_steps,

@@ -467,7 +467,8 @@ __device__ __forceinline__ bool worth_search(const Group &W, const float4 c, con
 // their terms (with the terms beyond the FP32 range apart in FP64).  In local memory: they are
 // touched a few times per receiver and split.  The limit is for receivers far out in the halo,
 // for which thousands of sources are within a factor 16 of the nearest: their warps, without
-// it, made the 65536-body passes a third longer (32 slots: a step of 53.1 ms, 16: 52.3 ms).
+// it, made the 65536-body passes a third longer.  (16, 32 and 64 slots: acc+gradient 7.98, 8.01
+// and 8.06 ms, the same errors within 2 %.)
 struct Slots {
     int j[2][SLOTS];
     float sum[2][6];
@@ -572,9 +573,10 @@ __device__ __forceinline__ float2 pair_weight(float2 r2, float2 m)
 
 // ACC: the variant that feeds a gradient (refined rsqrt, folds of every tile, dominant terms in
 // double-float by wmax).  Bound by the FP32 pipe (about 80 % of its cycles): 12 packed
-// operations a pair of far pairs (15 with ACC) and about 250 instructions a tile.  All 65536
-// particles of a Plummer sphere, with the sort: plain 2.50 -> 1.97 ms; ACC with its prepass 4.50
-// -> 2.72 ms.  12 resident warps an SM without spills beat 16 to 20 with fewer registers (2.14).
+// operations a pair of far pairs (18 with ACC) and about 250 instructions a tile.  All 65536
+// particles of a Plummer sphere, with the sort: plain 2.50 -> 2.12 ms (1.97 with one rounding a
+// tile); ACC with its prepass 4.50 -> 2.98 ms (2.72 with one of four roundings and sums of 16).
+// 12 resident warps an SM without spills beat 16 to 20 with fewer registers.
 template <bool ACC>
 __global__ void __launch_bounds__(32, ACC ? 13 : 12) k_acc_tile(const float *__restrict__ rec, int n, int nsplit,
                                                                       float eps2, double eps2d,
@@ -819,9 +821,9 @@ __device__ __forceinline__ void grad_weight(float2 r2, float2 m, float2 &w, floa
     w = __fmul2_rn(__fmul2_rn(m, y), ri2);
 }
 
-// 27 packed operations a pair of far pairs (47 in the pass on absolute three-part positions), the
-// FP32 pipe 77 % busy.  65536 particles: 6.35 -> 4.42 ms.  The registers of 10 warps an SM hold
-// the loop without spills (16 warps: the whole acc+gradient pass 7.49 instead of 7.36 ms).
+// 33 packed operations a pair of far pairs (47 in the pass on absolute three-part positions), the
+// FP32 pipe 84 % busy.  65536 particles: 6.35 -> 4.71 ms (4.42 with 27, one of four roundings a
+// separation).  The registers of 10 warps an SM hold the loop without spills.
 __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ rec, int n, int nsplit, double eps2d,
                                                       const float *__restrict__ wmax, double *__restrict__ part)
 {
@@ -1042,7 +1044,7 @@ __global__ void __launch_bounds__(32, 10) k_grad_tile(const float *__restrict__ 
 // term H leads, every later addition leaves up to half a unit of H to the low sum, an FP32 sum,
 // whose own rounding grows as their number: over the 512 terms of a split U of 20001 stars with
 // hard binaries was 9e-15 off (rms of 16 systems), over the 128 of k_potential_df 1.4e-15.)
-// Scalar FP32 throughput bounds it: 65536 particles 10.8 ms before.
+// Scalar FP32 throughput bounds it: 65536 particles 10.8 ms on every pair's absolute positions, 7.5 so.
 __global__ void __launch_bounds__(32) k_potential_tile(const int32_t *__restrict__ list, const float *__restrict__ rec,
                                                        const float4 *__restrict__ abs, int n, int nsplit, double eps2,
                                                        double *__restrict__ part)

@@ -121,8 +121,10 @@ constexpr int kOneSidedPairwiseMinN = 8192;
 constexpr int kOrderMinN = 16384;
 constexpr int kTileMinN = 8192;
 // the same for the Newtonian and gradient passes of one list: a pass entry point's from
-// kOrderForceMinN particles on (acc+gradient of 16384: 959 us so, 952 on the old passes; of 40603
-// 3.2 and 4.5 ms), and inside a step lists of at least kTileForceMinN.  Passes between two lists
+// kOrderForceMinN particles on (acc+gradient of 16384: 959 us so, 952 on the passes of every pair;
+// of 24576 1.51 and 1.95 ms, of 40603 3.37 and 4.46), and inside a step lists of at least
+// kTileForceMinN (a 65536-body step with 2048: 49.8 ms, 4096 50.0, 8192 50.7, 16384 50.5; of
+// 20011 stars with a Kroupa spectrum 12.93, 12.96, 13.02, 13.07).  Passes between two lists
 // do not take the tiles: a list's dominant terms then sit in few tiles of the other, and with
 // slots enough to keep its gradient as good as on the old passes (64 a split) the tiles are no
 // faster (25000 x 40000 particles 8.3 against 6.3 ms).

@@ -92,7 +92,9 @@ extern "C" void to_float(int n, const double *d, float *f) { for (int i = 0; i <
     f = np.ascontiguousarray(bits).view(np.float32)
     d = np.empty(f.size)
     lib.to_double(f.size, _p(f), _p(d))
-    assert np.array_equal(d, f.astype(np.float64), equal_nan=True) and np.array_equal(np.signbit(d), np.signbit(f))
+    with np.errstate(invalid="ignore"):
+        r = f.astype(np.float64)
+    assert np.array_equal(d, r, equal_nan=True) and np.array_equal(np.signbit(d), np.signbit(r))
 
     expo = np.concatenate([np.arange(880, 1170), [0, 1, 2046, 2047]]).astype(np.uint64)
     high = np.concatenate([[0, 1, 2, (1 << 23) - 2, (1 << 23) - 1], rng.integers(0, 1 << 23, 59)]).astype(np.uint64)
